@@ -50,7 +50,9 @@ constexpr int kStageA = BM * BK * 2;                   // 16 KB
 constexpr int kStageB = BN * BK * 2;                   // 32 KB
 constexpr int kStageBytes = kStageA + kStageB;
 constexpr int kTmemCols = 2 * BN;                      // two fp32 accumulators
-constexpr int kMaxSlices = 16;                         // 2 x slices partial lists per row (<= 32)
+constexpr int kSmCap = 160;                            // slices x row blocks never exceed this (nor the SM count)
+constexpr int kRoomyLists = 32;                        // partial lists per row that the workspace always has room for
+constexpr int kLaneLists = (2 * kSmCap + 31) / 32;     // partial lists per lane of the wide finishing kernel
 constexpr int kLmSmem = kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers, flags */;
 constexpr uint32_t kLmWaitLimit = 1u << 22;
 
@@ -506,7 +508,21 @@ struct ListLogits {
     }
 };
 
-// One warp per row: the row's P = 2 S partial lists are staged in shared
+// The merged list (entry m in lane m: key lk, token li, logit ll) and the smallest
+// key d left out of it: the row is finished by the streaming kernel's code.
+template <bool VERIFY>
+__device__ __forceinline__ void finish_merged(const RaceArgs& a, int64_t r, float lk, int li, float ll, float d, int kr,
+                                              int kp, int lane, int* s_tok, float* s_val) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) d = fminf(d, __shfl_xor_sync(FULL, d, o));
+    s_tok[lane] = li;
+    s_val[lane] = ll;
+    __syncwarp();
+    finalize_row_lp<0, VERIFY, false>(a, r, lk, li, d, kr, kp, lane, ListLogits{s_tok, s_val}, Blk{}, nullptr);
+    if constexpr (VERIFY) sequence_ticket(a, r, lane);
+}
+
+// One warp per row: the row's P = 2 S <= 32 partial lists are staged in shared
 // memory (list j in column j), merged by kp rounds of one warp argmin over the
 // list heads (as merge_rounds does for the streaming kernel), and the row is
 // finished by the streaming kernel's finishing code with the listed logits.
@@ -570,14 +586,75 @@ __global__ void __launch_bounds__(128) lmhead_finish_kernel(const RaceArgs a, co
             hl = h < kp ? s_l[w][h * 32 + lane] : 0.f;
         }
     }
-    float d = fminf(hk, th);
+    finish_merged<VERIFY>(a, r, lk, li, ll, fminf(hk, th), kr, kp, lane, s_tok[w], s_val[w]);
+}
+
+// The same for rows of more than 32 partial lists (few row blocks, many
+// slices): one one-warp CTA per row, lane j keeping the heads of lists j, j +
+// 32, ... in registers (all heads are loaded in one round trip).  Each of the
+// kp rounds takes the lane's smallest head and one warp argmin; only the
+// winning list's next entry is fetched (an L2 round trip, at most kp of them).
+// Tokens are unique across the lists of a row.
+template <bool VERIFY>
+__global__ void __launch_bounds__(32) lmhead_finish_wide_kernel(const RaceArgs a, const LmPartial* parts, int P) {
+    __shared__ int s_tok[32];
+    __shared__ float s_val[32];
+    const int lane = threadIdx.x;
+    const int64_t r = blockIdx.x;
+    int kr = 1;
+    if (!VERIFY) {
+        kr = a.row_k ? __ldg(a.row_k + r) : a.K;
+        kr = max(1, min(kr, a.K));
+    }
+    const int kp = min(kLmKP, kr + 2);
+    const LmPartial* Q = parts + (r * P + lane);
+    float hk[kLaneLists];
+    int hi[kLaneLists], h[kLaneLists];
+    float d = kInf;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d = fminf(d, __shfl_xor_sync(FULL, d, o));
-    s_tok[w][lane] = li;
-    s_val[w][lane] = ll;
-    __syncwarp();
-    finalize_row_lp<0, VERIFY, false>(a, r, lk, li, d, kr, kp, lane, ListLogits{s_tok[w], s_val[w]}, Blk{}, nullptr);
-    if constexpr (VERIFY) sequence_ticket(a, r, lane);
+    for (int j = 0; j < kLaneLists; ++j) {
+        const bool on = lane + 32 * j < P;
+        hk[j] = on ? __ldcg(Q[32 * j].key) : kInf;
+        hi[j] = on ? __ldcg(Q[32 * j].idx) : INT_MAX;
+        d = fminf(d, on ? __ldcg(&Q[32 * j].theta) : kInf);
+        h[j] = 0;
+    }
+    float lk = kInf, ll = 0.f;
+    int li = INT_MAX;
+    for (int m = 0; m < kp; ++m) {
+        float mk = kInf;
+        int mi = INT_MAX;
+#pragma unroll
+        for (int j = 0; j < kLaneLists; ++j)
+            if (lex_less(hk[j], hi[j], mk, mi)) {
+                mk = hk[j];
+                mi = hi[j];
+            }
+        float bk;
+        const int bi = warp_argmin(mk, mi, bk);
+        if (bi == INT_MAX) break;  // fewer listed entries than kp (warp-uniform)
+        float won = 0.f;
+        if (mi == bi) {
+#pragma unroll
+            for (int j = 0; j < kLaneLists; ++j)
+                if (hi[j] == bi) {
+                    const LmPartial* L = Q + 32 * j;
+                    won = __ldcg(L->logit + h[j]);
+                    ++h[j];
+                    hk[j] = h[j] < kp ? __ldcg(L->key + h[j]) : kInf;
+                    hi[j] = h[j] < kp ? __ldcg(L->idx + h[j]) : INT_MAX;
+                }
+        }
+        won = __shfl_sync(FULL, won, __ffs(__ballot_sync(FULL, mi == bi)) - 1);
+        if (lane == m) {
+            lk = bk;
+            li = bi;
+            ll = won;
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < kLaneLists; ++j) d = fminf(d, hk[j]);
+    finish_merged<VERIFY>(a, r, lk, li, ll, d, kr, kp, lane, s_tok, s_val);
 }
 
 // ---------------------------------------------------------------- host side
@@ -623,21 +700,25 @@ static cudaError_t launch_gemm(const CUtensorMap& tA, const CUtensorMap& tB, con
     return cudaGetLastError();
 }
 
-// the schedule: MB row blocks x S vocabulary slices, S = SMs / MB (1..kMaxSlices, <= NT)
+// The schedule: MB row blocks x S vocabulary slices, S = SMs / MB (at least 1, at most NT), so that
+// every SM has a CTA.  With few row blocks the pass is bound by reading the weights once from HBM,
+// which takes the whole chip: the two launches of one sequence (41 rows of d = 4096, 33 of d = 2048,
+// V = 128256: 1.58 GB) take 317 us = 5.0 TB/s on 152 slices, 1131 us on 16.
 static void schedule(LmArgs& a) {
     a.MB = (int)((a.n_rows + BM - 1) / BM);
     a.NT = (int)((a.V + BN - 1) / BN);
     a.KB = (int)((a.d + BK - 1) / BK);
-    int S = device_sm_count() / max(1, a.MB);
-    S = max(1, min(S, kMaxSlices));
-    a.S = min(S, a.NT);
+    a.S = min(max(1, min(device_sm_count(), kSmCap) / max(1, a.MB)), a.NT);
 }
 
 }  // namespace lm
 
+// n_rows x 2 S partial lists: at most 2 BM kSmCap of them, or 2 per row beyond kSmCap row blocks.
+// The size never falls as n_rows grows, so a workspace serves every smaller call too.
 size_t lmhead_workspace_bytes(int64_t n_rows, int32_t n_seq) {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    return al(sizeof(lm::LmPartial) * 2 * lm::kMaxSlices * (size_t)n_rows) + al(sizeof(uint32_t) * (size_t)(n_seq > 0 ? n_seq : 0));
+    const size_t lists = (size_t)max((int64_t)2 * lm::BM * lm::kSmCap, n_rows * lm::kRoomyLists);
+    return al(sizeof(lm::LmPartial) * lists) + al(sizeof(uint32_t) * (size_t)(n_seq > 0 ? n_seq : 0));
 }
 
 cudaError_t launch_lmhead_logits(const void* hidden, int64_t ldh, const void* weight, int64_t ldw, int64_t n_rows,
@@ -679,6 +760,13 @@ cudaError_t launch_lmhead_race(const void* hidden, int64_t ldh, const void* weig
                              : lm::launch_gemm<lm::RaceEpi<lm::kLmKP>>(tA, tB, a, st);
     if (e != cudaSuccess) return e;
     const int P = 2 * a.S;
+    if (P > 32) {
+        if (verify)
+            lm::lmhead_finish_wide_kernel<true><<<(unsigned)ra.n_rows, 32, 0, st>>>(ra, a.partials, P);
+        else
+            lm::lmhead_finish_wide_kernel<false><<<(unsigned)ra.n_rows, 32, 0, st>>>(ra, a.partials, P);
+        return cudaGetLastError();
+    }
     const unsigned blocks = (unsigned)((ra.n_rows + 3) / 4);
     if (verify)
         lm::lmhead_finish_kernel<true><<<blocks, 128, 0, st>>>(ra, a.partials, P);

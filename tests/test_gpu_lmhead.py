@@ -190,6 +190,28 @@ def test_fused_race_matches_the_oracle_on_dyadic_operands():
         np.testing.assert_allclose(v["score_sum"].cpu().numpy(), ow["score_sum"], rtol=1e-5)
 
 
+# row blocks of 128 rows x vocabulary slices of 256-column tiles over the SMs: one row on every
+# slice, a whole and a just begun second block, fewer tiles than SMs (one tile a slice, the last one
+# ragged), and both sides of 32 partial lists per row (9 and 10 blocks: 16 and 15 slices on 152 SMs)
+@pytest.mark.parametrize("n,V", [(1, 39000), (41, 38913), (128, 700), (129, 20000), (520, 9001), (1030, 6000),
+                                 (1153, 6000)])
+def test_fused_race_over_many_slices_equals_the_unfused_path(n, V):
+    h, w = _normal(n, V, 72, n + V)
+    _, (key, ctx, pos) = _ids(n, n)
+    logits = pps.lmhead_logits(h, w)
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for K, mode in ((1, pps.DISTINCT), (8, pps.IID)):
+        fused = pps.lmhead_draft_list(h, w, key, ctx, pos, K, mode=mode, status=st)
+        _assert_same(fused, pps.draft_list(logits, key, ctx, pos, K, mode=mode, status=st), DRAFT)
+    off = torch.arange(n + 1, dtype=torch.int32, device="cuda")  # every row a tree of one node
+    none = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    one = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    args = (1, off, none, one, one[0], one)
+    v = pps.lmhead_verify_tree(h, w, key, ctx, pos, *args, status=st)
+    _assert_same(v, pps.verify_tree(logits, key, ctx, pos, *args, status=st), VERIFY)
+    assert int(st.item()) == 0
+
+
 def test_full_size_lmhead_workload_every_row():
     # the benchmark's LM-head workload: the K = 8 chain tree of 64 sequences, V = 128256, target
     # d = 4096 (2624 node rows), draft d = 2048 (2112 draft rows); fused against unfused everywhere
