@@ -5,6 +5,7 @@ fallback: a missing or unloadable libpps.so raises immediately.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 import threading
@@ -66,6 +67,9 @@ def philox_rounds() -> int:
 def lib():
     """Load libpps.so (raises if it was not built)."""
     global _lib
+    loaded = _lib
+    if loaded is not None:
+        return loaded
     with _lock:
         if _lib is None:
             if not os.path.exists(LIB_PATH):
@@ -151,24 +155,38 @@ def _check(fn, code):
         raise PPSError(fn, code)
 
 
+# Host cost of a call.  A step of few rows runs two launches of about 20 us, and its two calls took
+# 47 us of Python (tensor checks 14, stream object 4, device guard 3, ids 4, pointer objects 6), so
+# the binding keeps every check but makes the common outcome cheap: one expression per tensor, raw
+# pointers and stream handles instead of wrapper objects, and a device switch only when it is needed.
+
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream, dev=None):
     """The stream's handle; with no stream, the current stream of `dev` (the tensors' device)."""
     if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    elif dev is not None and stream.device != dev:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if dev is None else dev.index)
+    if dev is not None and stream.device != dev:
         raise ValueError(f"stream is on {stream.device}, the tensors on {dev}")
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
+
+
+_HERE_ALREADY = contextlib.nullcontext()
+
+
+def _on(dev):
+    """A context in which `dev` is the current device."""
+    return _HERE_ALREADY if torch.cuda.current_device() == dev.index else torch.cuda.device(dev)
 
 
 def _need(name, t, dev, dtype, numel=0, contiguous=True):
     """Raise unless tensor `t` (skipped when None) is on `dev` with `dtype` and holds at least
     `numel` elements: the library writes and reads through plain pointers, so a short or
     misplaced buffer must be refused here, before anything is launched."""
-    if t is None:
+    if t is None or (isinstance(t, torch.Tensor) and t.is_cuda and t.get_device() == dev.index and t.dtype is dtype
+                     and t.numel() >= numel and (not contiguous or t.is_contiguous())):
         return
     if not isinstance(t, torch.Tensor) or not t.is_cuda or t.device != dev:
         raise TypeError(f"{name} must be a CUDA tensor on {dev}")
@@ -191,9 +209,10 @@ def _dtype_code(t: torch.Tensor) -> int:
 def _ids(key, ctx, pos, n=0, dev=None):
     """Row ids (bit patterns of the unsigned key, context label and position), n of each."""
     for name, t, dt in (("key", key, torch.int64), ("ctx", ctx, torch.int64), ("pos", pos, torch.int32)):
-        if not t.is_cuda or t.dtype != dt or not t.is_contiguous():
+        if not t.is_cuda or t.dtype is not dt or not t.is_contiguous():
             raise TypeError(f"{name} must be a contiguous CUDA {dt} tensor (bit pattern of the unsigned id)")
-        _need(name, t, dev if dev is not None else t.device, dt, n)
+        if (dev is not None and t.get_device() != dev.index) or t.numel() < n:
+            _need(name, t, dev if dev is not None else t.device, dt, n)
     return RowIds(key.data_ptr(), ctx.data_ptr(), pos.data_ptr())
 
 
@@ -220,7 +239,7 @@ def workspace(n_rows: int, n_seq: int = 0, device=None) -> torch.Tensor:
 
 def workspace_clear(ws: torch.Tensor, stream=None):
     _need("ws", ws, ws.device, torch.uint8)
-    with torch.cuda.device(ws.device):
+    with _on(ws.device):
         _check("pps_workspace_clear", lib().pps_workspace_clear(_ptr(ws), ws.numel(), _stream(stream, ws.device)))
 
 
@@ -251,7 +270,7 @@ def draft_list(q_logits, key, ctx, pos, K: int, row_k=None, mode: int = DISTINCT
     _need_draft(out, n, K, row_k, status, dev)
     _need("ws", ws, dev, torch.uint8)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         if top_k > 0:
             code = lib().pps_draft_list_trunc(_ptr(q_logits), _dtype_code(q_logits), n, V, stride, ids,
                                               float(temperature), int(top_k), float(top_p), int(K), _ptr(row_k),
@@ -283,7 +302,7 @@ def draft_list_noalloc(q_logits, key, ctx, pos, K: int, row_k=None, mode: int = 
                    samples=torch.empty(n, K, dtype=torch.int32, device=dev) if samples else None)
     _need_draft(out, n, K, row_k, status, dev)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_draft_list_noalloc(_ptr(q_logits), _dtype_code(q_logits), n, V, stride, ids,
                                             float(temperature), int(K), _ptr(row_k), int(mode), _ptr(out["tok"]),
                                             _ptr(out.get("key")), _ptr(out["mult"]), _ptr(out["ndist"]),
@@ -323,7 +342,7 @@ def verify_tree(p_logits, key, ctx, pos, gamma: int, seq_off, node_draft_row, dr
     _need("status", status, dev, torch.int32, 1)
     _need("ws", ws, dev, torch.uint8)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         if top_k > 0:
             code = lib().pps_verify_tree_trunc(_ptr(p_logits), _dtype_code(p_logits), n, V, stride, ids,
                                                float(temperature), int(top_k), float(top_p), n_seq, int(gamma),
@@ -367,7 +386,7 @@ def wm_score(tokens, key, ctx, pos, seg_off=None, out_score=None, out_sum=None, 
     _need("out_score", out_score, dev, torch.float32, n)
     _need("out_sum", out_sum, dev, torch.float64, n_seg)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_wm_score(_ptr(tokens), ids, n, n_seg, _ptr(seg_off), _ptr(out_score), _ptr(out_sum),
                                   _stream(stream, dev))
     _check("pps_wm_score", code)
@@ -382,7 +401,7 @@ def tree_expand(K: int, gamma: int, depth: int, draft, rows_key, rows_ctx, rows_
     n_seq = nxt["k"].numel() // K
     dev = nxt["k"].device
     ids = _ids(rows_key, rows_ctx, rows_pos, 0, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_tree_expand(n_seq, int(K), int(gamma), int(depth), _ptr(draft["tok"]), _ptr(draft["mult"]),
                                      _ptr(draft["ndist"]), ids, _ptr(row_k), _ptr(nxt["key"]), _ptr(nxt["ctx"]),
                                      _ptr(nxt["pos"]), _ptr(nxt["k"]), _ptr(child_node), _ptr(nodes["key"]),
@@ -409,7 +428,7 @@ def draft_hetero(q_logits, key, ctx, pos, row_block, n_blocks: int, temperature:
     _need("status", status, dev, torch.int32, 1)
     _need("ws", ws, dev, torch.uint8)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         if top_k > 0:
             code = lib().pps_draft_hetero_trunc(_ptr(q_logits), _dtype_code(q_logits), n, V, stride, ids,
                                                 float(temperature), int(top_k), float(top_p), _ptr(row_block),
@@ -434,7 +453,7 @@ def hetero_expand(n_blocks: int, gamma: int, depth: int, draft_tok, rows_key, ro
     nx = nxt or {}
     dev = row_owner.device
     ids = _ids(rows_key, rows_ctx, rows_pos, 0, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_hetero_expand(n_seq, int(n_blocks), int(gamma), int(depth), _ptr(draft_tok), ids,
                                        _ptr(row_owner), _ptr(nx.get("key")), _ptr(nx.get("ctx")), _ptr(nx.get("pos")),
                                        _ptr(nx.get("owner")), _ptr(lists["tok"]), _ptr(lists["ndist"]),
@@ -452,7 +471,7 @@ def hetero_block(tokens, key, ctx, pos, n_blocks: int, out=None, stream=None):
     _need_detector(tokens, None, n, 0, dev)
     _need("out", out, dev, torch.int32, n)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_hetero_block(_ptr(tokens), ids, n, int(n_blocks), _ptr(out), _stream(stream, dev))
     _check("pps_hetero_block", code)
     return out
@@ -472,7 +491,7 @@ def wm_detect(tokens, key, ctx, pos, seg_off=None, kind: int = SCORE_AARONSON, p
     out_logp = torch.empty(n_seg, dtype=torch.float64, device=dev) if want_logp else None
     _need_detector(tokens, seg_off, n, n_seg, dev)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_wm_detect(_ptr(tokens), ids, n, n_seg, _ptr(seg_off), int(kind), float(param),
                                    _ptr(out_score), _ptr(out_sum), _ptr(out_logp), _stream(stream, dev))
     _check("pps_wm_detect", code)
@@ -484,7 +503,7 @@ def philox_words(key, ctx, pos, vocab: int, arrival: int = 1, stream=None):
     dev = key.device
     out = torch.empty(n, vocab, dtype=torch.int32, device=dev)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         _check("pps_philox_words", lib().pps_philox_words(ids, n, vocab, arrival, _ptr(out), _stream(stream, dev)))
     return out
 
@@ -541,7 +560,7 @@ def lmhead_logits(hidden, weight, out=None, stream=None):
     if out.dtype != torch.float32 or out.device != dev or out.dim() != 2 or out.stride(1) != 1 or \
             out.shape[0] < n or out.shape[1] < V:
         raise TypeError("out must be a float32 [n_rows, >= vocab] tensor on the operands' device")
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_lmhead_logits(_ptr(hidden), ldh, _ptr(weight), ldw, n, V, d, _ptr(out), out.stride(0),
                                        _stream(stream, dev))
     _check("pps_lmhead_logits", code)
@@ -565,7 +584,7 @@ def lmhead_draft_list(hidden, weight, key, ctx, pos, K: int, row_k=None, mode: i
     _need_draft(out, n, K, row_k, status, dev)
     _need("ws", ws, dev, torch.uint8)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_lmhead_draft_list(_ptr(hidden), ldh, _ptr(weight), ldw, n, V, d, ids, float(temperature),
                                            int(K), _ptr(row_k), int(mode), _ptr(out["tok"]), _ptr(out.get("key")),
                                            _ptr(out["mult"]), _ptr(out["ndist"]), _ptr(out.get("samples")),
@@ -604,7 +623,7 @@ def lmhead_verify_tree(hidden, weight, key, ctx, pos, gamma: int, seq_off, node_
     _need("status", status, dev, torch.int32, 1)
     _need("ws", ws, dev, torch.uint8)
     ids = _ids(key, ctx, pos, n, dev)
-    with torch.cuda.device(dev):
+    with _on(dev):
         code = lib().pps_lmhead_verify_tree(_ptr(hidden), ldh, _ptr(weight), ldw, n, V, d, ids, float(temperature),
                                             n_seq, int(gamma), _ptr(seq_off), _ptr(node_draft_row), n_draft,
                                             _ptr(draft_tok), _ptr(draft_ndist), int(K), _ptr(child_node),

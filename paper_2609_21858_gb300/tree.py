@@ -54,6 +54,12 @@ class TreeBuilder:
         self.row_k = torch.zeros(self.row_key.numel(), **i32)
         self.roots = self.seq_off[:-1].long()
         self.ws = pps.workspace(n_seq * K, 0, dev)
+        # what every run hands on per depth, and the root nodes' identities, as views made once
+        self._ids = [tuple(t[self.rows(d)] for t in (self.row_key, self.row_ctx, self.row_pos, self.row_k))
+                     for d in range(gamma + 1)]
+        self._out = [dict(tok=self.draft_tok[s], key=None, mult=self.draft_mult[s], ndist=self.draft_ndist[s],
+                          samples=None) for s in map(self.rows, range(gamma))]
+        self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
 
     def rows(self, d: int) -> slice:
         return slice(self.depth_start[d], self.depth_start[d] + self.n_seq * self.width[d])
@@ -62,20 +68,18 @@ class TreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_list (IID) and one pps_tree_expand."""
         K = self.K
-        s0 = self.rows(0)
-        self.row_key[s0], self.row_ctx[s0], self.row_pos[s0] = root_key, root_ctx, root_pos
-        self.row_k[s0] = K
-        self.node_key[self.roots], self.node_ctx[self.roots], self.node_pos[self.roots] = root_key, root_ctx, root_pos
+        for mine, root, x in zip(self._ids[0], self._root, (root_key, root_ctx, root_pos)):
+            mine.copy_(x)
+            root.copy_(x)
+        self._ids[0][3].fill_(K)
+        nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
         for d in range(self.gamma):
-            s, sn = self.rows(d), self.rows(d + 1)
-            key, ctx, pos, k = self.row_key[s], self.row_ctx[s], self.row_pos[s], self.row_k[s]
-            out = dict(tok=self.draft_tok[s], key=None, mult=self.draft_mult[s], ndist=self.draft_ndist[s],
-                       samples=None)
+            key, ctx, pos, k = self._ids[d]
+            out = self._out[d]
             pps.draft_list(draft_logits(d, key, ctx, pos), key, ctx, pos, K, row_k=k, mode=pps.IID,
                            temperature=temperature, ws=self.ws, out=out, top_k=top_k, top_p=top_p, stream=stream)
-            nxt = dict(key=self.row_key[sn], ctx=self.row_ctx[sn], pos=self.row_pos[sn], k=self.row_k[sn])
-            pps.tree_expand(K, self.gamma, d, out, key, ctx, pos, k, nxt, self.child_node,
-                            dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos), stream=stream)
+            nxt = dict(zip(("key", "ctx", "pos", "k"), self._ids[d + 1]))
+            pps.tree_expand(K, self.gamma, d, out, key, ctx, pos, k, nxt, self.child_node, nodes, stream=stream)
         return self
 
     def verify(self, p_logits, temperature: float = 1.0, top_k: int = 0, top_p: float = 1.0, ws=None, out=None,
@@ -136,6 +140,10 @@ class HeteroTreeBuilder:
         self.draft_tok = torch.full((nr,), -1, **i32)
         self.roots = self.seq_off[:-1].long()
         self.ws = pps.workspace(n_seq * B, 0, dev)
+        self._ids = [tuple(t[self.rows(d)] for t in (self.row_key, self.row_ctx, self.row_pos, self.row_owner))
+                     for d in range(gamma)]
+        self._blk_tok = [(self.row_block[s], self.draft_tok[s]) for s in map(self.rows, range(gamma))]
+        self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
 
     def rows(self, d: int) -> slice:
         n = self.n_seq * self.B
@@ -145,25 +153,19 @@ class HeteroTreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_hetero and one pps_hetero_expand."""
         B = self.B
-        s0 = self.rows(0)
-        self.row_key[s0] = root_key.repeat_interleave(B)
-        self.row_ctx[s0] = root_ctx.repeat_interleave(B)
-        self.row_pos[s0] = root_pos.repeat_interleave(B)
-        self.row_owner[s0] = 0
-        self.node_key[self.roots], self.node_ctx[self.roots], self.node_pos[self.roots] = root_key, root_ctx, root_pos
+        for mine, root, x in zip(self._ids[0], self._root, (root_key, root_ctx, root_pos)):
+            mine.view(self.n_seq, B).copy_(x[:, None].expand(-1, B))
+            root.copy_(x)
+        self._ids[0][3].zero_()
         lists = dict(tok=self.list_tok, ndist=self.list_nd, child=self.child_node)
         nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
         for d in range(self.gamma):
-            s = self.rows(d)
-            key, ctx, pos, blk = self.row_key[s], self.row_ctx[s], self.row_pos[s], self.row_block[s]
+            key, ctx, pos, owner = self._ids[d]
+            blk, tok = self._blk_tok[d]
             pps.draft_hetero(draft_logits(d, key, ctx, pos, blk), key, ctx, pos, blk, B, temperature=temperature,
-                             ws=self.ws, out_tok=self.draft_tok[s], stream=stream, top_k=top_k, top_p=top_p)
-            nxt = None
-            if d + 1 < self.gamma:
-                sn = self.rows(d + 1)
-                nxt = dict(key=self.row_key[sn], ctx=self.row_ctx[sn], pos=self.row_pos[sn], owner=self.row_owner[sn])
-            pps.hetero_expand(B, self.gamma, d, self.draft_tok[s], key, ctx, pos, self.row_owner[s], nxt, lists,
-                              nodes, stream=stream)
+                             ws=self.ws, out_tok=tok, stream=stream, top_k=top_k, top_p=top_p)
+            nxt = dict(zip(("key", "ctx", "pos", "owner"), self._ids[d + 1])) if d + 1 < self.gamma else None
+            pps.hetero_expand(B, self.gamma, d, tok, key, ctx, pos, owner, nxt, lists, nodes, stream=stream)
         return self
 
     def verify(self, p_logits, temperature: float = 1.0, top_k: int = 0, top_p: float = 1.0, ws=None, out=None,
