@@ -208,11 +208,10 @@ __device__ __forceinline__ float key32(uint32_t w, float l, float c) {
     return k != k ? __int_as_float(0x7f800000) : k;
 }
 
-// fp64 race key s = ln E - l / T (the paper's definition, used for near-ties)
-__device__ __forceinline__ double exp1_f64(uint32_t w) {
-    if (w < 0x80000000u) return -log(((double)w + 0.5) * 0x1p-32);
-    return -log1p(-(((double)(~w) + 0.5) * 0x1p-32));
-}
+// fp64 race key s = ln E - l / T (the paper's definition, used for near-ties).
+// u = (w + 1/2) 2^-32 has 33 significant bits, so it is exact in fp64 for every
+// w, also next to 1, and one logarithm of it is as accurate as log1p(-(1 - u)).
+__device__ __forceinline__ double exp1_f64(uint32_t w) { return -log(((double)w + 0.5) * 0x1p-32); }
 __device__ __forceinline__ double key64(uint32_t w, float l, float T) {
     double ld = (double)l;
     if (ld != ld) return __longlong_as_double(0x7ff0000000000000ll);
@@ -295,10 +294,8 @@ static __device__ __noinline__ float block_key_of(uint64_t key, uint64_t ctx, ui
 // so A = ln 2 * neg_log2_u(~w).  The transform's relative error is below
 // 2^kErrAbs - 1 < 2.1e-6 for every word (pps_selftest_key_error checks all
 // 2^32), 2.2e-6 with the final product; its absolute error is below 2e-7.
-__device__ __forceinline__ double score64(uint32_t w) {
-    if (w < 0x80000000u) return -log1p(-(((double)w + 0.5) * 0x1p-32));
-    return -log(((double)(~w) + 0.5) * 0x1p-32);
-}
+// In fp64 1 - u is exact too, so its logarithm is taken as it stands.
+__device__ __forceinline__ double score64(uint32_t w) { return exp1_f64(~w); }
 __device__ __forceinline__ float score32(uint32_t w) { return 0.69314718055994531f * neg_log2_u(~w); }
 
 // Detection score kinds of the pivot r = u (App. D): Aaronson -ln(1 - r), the

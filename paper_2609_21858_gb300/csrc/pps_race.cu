@@ -99,6 +99,21 @@ __device__ __forceinline__ uint32_t ord_key(float f) {
 __device__ __forceinline__ float unord_key(uint32_t u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
+// smallest of the warp's values (none NaN)
+__device__ __forceinline__ float warp_min(float f) { return unord_key(__reduce_min_sync(FULL, ord_key(f))); }
+// the k-th smallest of the warp's 32 values (none NaN): the smallest by one
+// redux.min, others bit by bit
+__device__ __forceinline__ float warp_kth(float f, int k) {
+    if (k == 1) return warp_min(f);
+    const uint32_t u = ord_key(f);
+    uint32_t res = 0;
+#pragma unroll 1
+    for (int b = 31; b >= 0; --b) {
+        const uint32_t cand = res | (1u << b);
+        if (__popc(__ballot_sync(FULL, u < cand)) < k) res = cand;
+    }
+    return unord_key(res);
+}
 // Warp argmin of (key, token) by lexicographic order; tokens are non-negative
 // (INT_MAX: empty).  Returns the winning token (INT_MAX when every lane is
 // empty) and its key in bk.
@@ -139,11 +154,15 @@ __device__ __forceinline__ float list_insert(float& lk, int& li, float ck, int c
     return last;
 }
 
-// bitonic sort of one entry per lane, ascending
+// bitonic sort of one entry per lane, ascending.  Rolled: the sorts, merges and
+// row finishes run a few times per row, and a launch of few rows waits for
+// their instructions to be fetched (no-instruction stalls were the largest of
+// a one-sequence launch: 2.5 of 8 per issue), so this code is kept short (a step of
+// 8 sequences of 4 chains, V = 32000: 58.3 -> 54.9 us).
 __device__ __forceinline__ void warp_sort(float& k, int& i, int lane) {
-#pragma unroll
+#pragma unroll 1
     for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
+#pragma unroll 1
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
             float ok = __shfl_xor_sync(FULL, k, stride);
             int oi = __shfl_xor_sync(FULL, i, stride);
@@ -172,7 +191,7 @@ __device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi
         li = ri;
     }
     // (lk, li) is now bitonic and holds the 32 smallest of the union
-#pragma unroll
+#pragma unroll 1
     for (int stride = 16; stride > 0; stride >>= 1) {
         float xk = __shfl_xor_sync(FULL, lk, stride);
         int xi = __shfl_xor_sync(FULL, li, stride);
@@ -185,8 +204,7 @@ __device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi
     }
     if (TRACK) {
         if (kp < 32) dropk = fminf(dropk, __shfl_sync(FULL, lk, kp & 31));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) dropk = fminf(dropk, __shfl_xor_sync(FULL, dropk, o));
+        dropk = warp_min(dropk);
     }
     if (lane >= kp) {
         lk = kInf;
@@ -196,9 +214,9 @@ __device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi
 }
 
 __device__ __forceinline__ void warp_sort_d(double& k, int& i, int lane) {
-#pragma unroll
+#pragma unroll 1
     for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
+#pragma unroll 1
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
             double ok = __shfl_xor_sync(FULL, k, stride);
             int oi = __shfl_xor_sync(FULL, i, stride);
@@ -385,11 +403,7 @@ __device__ __forceinline__ void offer_survivors(WarpList& L, float (&pk)[VW], in
     float rem = kInf;
 #pragma unroll
     for (int e = 0; e < VW; ++e) rem = fminf(rem, pk[e]);
-    if (L.tight() && __any_sync(FULL, rem < kInf)) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) rem = fminf(rem, __shfl_xor_sync(FULL, rem, o));
-        L.mr = fminf(L.mr, rem);
-    }
+    if (L.tight() && __any_sync(FULL, rem < kInf)) L.mr = fminf(L.mr, warp_min(rem));
 }
 
 // Filter, key and offer the 4 tokens of one Philox block (counter cb, tokens
@@ -547,13 +561,14 @@ __device__ __noinline__ float seed_theta(const char* row, int64_t v0, float c, u
     const uint32_t cl = DT == 1 ? (uint32_t)(2 * (v0 + lane)) : (uint32_t)(v0 + lane);
     float bk = kInf;
     int bi = INT_MAX;
-#pragma unroll
+#pragma unroll 1
     for (int b = 0; b < 2; ++b) {
-        const uint32_t cb = cl + block_offset<DT>(b);
+        const uint32_t cb = cl + (b ? block_offset<DT>(1) : 0u);
         const uint4 q = rp.block(cb);
         const uint32_t wq[4] = {q.x, q.y, q.z, q.w};
         float l[4];
-        block_logits<DT>(d, b, l);
+        block_logits<DT>(d, 0, l);
+        d[0] = DT == 1 ? make_uint4(d[0].z, d[0].w, 0u, 0u) : d[1];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             const float k = key32(wq[e], l[e], c);
@@ -567,8 +582,7 @@ __device__ __noinline__ float seed_theta(const char* row, int64_t v0, float c, u
     if constexpr (BLK)
         bk = block_key_of(key, ctx, pos, bi, word_of(key, ctx, pos, bi, 1), load_logit<DT>(row, bi), c, blk.b,
                           blk.B, blk.invB());
-    warp_sort(bk, bi, lane);
-    return filter_slack(__shfl_sync(FULL, bk, k - 1)) + (BLK ? 4.0f * kBlkErr : 0.f);
+    return filter_slack(warp_kth(bk, k)) + (BLK ? 4.0f * kBlkErr : 0.f);
 }
 
 // ---------------------------------------------------------------- the fast loop
@@ -953,9 +967,7 @@ __device__ __noinline__ bool iid_fast(const RaceArgs& a, int64_t r, float lk, in
             }
         }
     }
-    float nxt = h;  // the best unselected score
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) nxt = fminf(nxt, __shfl_xor_sync(FULL, nxt, off));
+    const float nxt = warp_min(h);  // the best unselected score
     const float after = __shfl_down_sync(FULL, selh, 1);
     const float b = lane + 1 < nsel ? after : nxt;
     const bool bad = lane < nsel && b < kInf &&
@@ -1262,21 +1274,20 @@ __device__ __noinline__ void walk_sequence(const RaceArgs& a, int s, int lane) {
         const uint32_t w = __ldcg(a.out_word + c);
         if (y >= 0) keep(y, w);
     }
-    // scores of the emitted tokens, their sum in emission order
-    double A[3];
+    // scores of the emitted tokens, their sum in emission order (one round for gamma < 32)
     double S = 0.0;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        const int t = q * 32 + lane;
-        A[q] = t < ne ? score64(w_[q]) : 0.0;
+#pragma unroll 1
+    for (int q = 0; 32 * q < W; ++q) {
+        const int t = 32 * q + lane;
+        const int y = q == 0 ? y_[0] : q == 1 ? y_[1] : y_[2];
+        const uint32_t w = q == 0 ? w_[0] : q == 1 ? w_[1] : w_[2];
+        const double A = t < ne ? score64(w) : 0.0;
         if (t < W) {
-            a.out_em[(size_t)s * W + t] = t < ne ? y_[q] : -1;
-            a.out_sc[(size_t)s * W + t] = (float)A[q];
+            a.out_em[(size_t)s * W + t] = t < ne ? y : -1;
+            a.out_sc[(size_t)s * W + t] = (float)A;
         }
-    }
-    for (int t = 0; t < ne; ++t) {
-        const int q = t >> 5;
-        S += __shfl_sync(FULL, q == 0 ? A[0] : (q == 1 ? A[1] : A[2]), t & 31);
+#pragma unroll 1
+        for (int m = 0; m < 32 && 32 * q + m < ne; ++m) S += __shfl_sync(FULL, A, m);
     }
     if (lane == 0) {
         a.out_acc[s] = acc;
@@ -1402,10 +1413,7 @@ __device__ __noinline__ void merge_rounds(const RaceArgs& a, int64_t r, int64_t 
             hi = h < kp ? s_i[lane * 32 + h] : INT_MAX;
         }
     }
-    float d = fminf(hk, th);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) d = fminf(d, __shfl_xor_sync(FULL, d, o));
-    theta_drop = fminf(theta_drop, d);
+    theta_drop = fminf(theta_drop, warp_min(fminf(hk, th)));
     __syncwarp();
 }
 
