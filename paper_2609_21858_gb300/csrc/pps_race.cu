@@ -2,7 +2,7 @@
 // target winners) with the tree walk fused behind a per-sequence ticket.
 //
 // Work split.  The n_rows x vocab logits are viewed as one flattened range of
-// 16-byte vectors (8 bf16 or 4 fp32 tokens).  A CTA is a single warp; warp gw
+// 16-byte vectors (8 bf16 or 4 fp32 tokens; not necessarily aligned, load_vec).  A CTA is a single warp; warp gw
 // of NW streams the slice [gw*total/NW, (gw+1)*total/NW), i.e. a few whole
 // rows plus at most two partial rows.  A row cut between warps is merged and
 // finished by the warp that arrives last at the row's counter; a sequence's
@@ -37,9 +37,6 @@
 #endif
 #ifndef PPS_UNITS_VERIFY
 #define PPS_UNITS_VERIFY 3  // the same for verify rows and one-token draft rows
-#endif
-#ifndef PPS_PREFETCH
-#define PPS_PREFETCH 0  // 1: load the next iteration's vectors one iteration ahead (costs registers)
 #endif
 #ifndef PPS_ROWBOUND
 #define PPS_ROWBOUND 1  // 1: warps that share a row share its filter bound through the workspace
@@ -129,36 +126,10 @@ __device__ __forceinline__ int warp_argmin(float k, int t, float& bk) {
 // A warp list holds entries (k, i) sorted ascending by (k, i), entry m in
 // lane m; lanes >= kp hold (+inf, INT_MAX).
 
-// insert one warp-uniform entry (serial path for a few survivors); returns
-// the key left out: the entry pushed out of a full list (+inf if there was
-// room), or ck itself when it does not enter
-__device__ __forceinline__ float list_insert(float& lk, int& li, float ck, int ci, int kp, int lane) {
-    bool less = lane < kp && lex_less(ck, ci, lk, li);
-    unsigned m = __ballot_sync(FULL, less);
-    if (m == 0) return ck;
-    const float last = __shfl_sync(FULL, lk, kp - 1);
-    int p = __ffs(m) - 1;
-    float uk = __shfl_up_sync(FULL, lk, 1);
-    int ui = __shfl_up_sync(FULL, li, 1);
-    if (lane > p) {
-        lk = uk;
-        li = ui;
-    } else if (lane == p) {
-        lk = ck;
-        li = ci;
-    }
-    if (lane >= kp) {
-        lk = kInf;
-        li = INT_MAX;
-    }
-    return last;
-}
-
 // bitonic sort of one entry per lane, ascending.  Rolled: the sorts, merges and
 // row finishes run a few times per row, and a launch of few rows waits for
 // their instructions to be fetched (no-instruction stalls were the largest of
-// a one-sequence launch: 2.5 of 8 per issue), so this code is kept short (a step of
-// 8 sequences of 4 chains, V = 32000: 58.3 -> 54.9 us).
+// a one-sequence launch), so this code is kept short.
 __device__ __forceinline__ void warp_sort(float& k, int& i, int lane) {
 #pragma unroll 1
     for (int size = 2; size <= 32; size <<= 1) {
@@ -180,7 +151,6 @@ __device__ __forceinline__ void warp_sort(float& k, int& i, int lane) {
 
 // merge a sorted list (lk, li) with a sorted batch (ok, oi); keep the kp smallest.
 // Returns (warp-uniform) the smallest key it discards: the (kp+1)-th of the union.
-template <bool TRACK>
 __device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi, int kp, int lane) {
     float rk = __shfl_sync(FULL, ok, 31 - lane);
     int ri = __shfl_sync(FULL, oi, 31 - lane);
@@ -202,10 +172,8 @@ __device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi
             li = xi;
         }
     }
-    if (TRACK) {
-        if (kp < 32) dropk = fminf(dropk, __shfl_sync(FULL, lk, kp & 31));
-        dropk = warp_min(dropk);
-    }
+    if (kp < 32) dropk = fminf(dropk, __shfl_sync(FULL, lk, kp & 31));
+    dropk = warp_min(dropk);
     if (lane >= kp) {
         lk = kInf;
         li = INT_MAX;
@@ -269,6 +237,49 @@ __device__ __forceinline__ uint4 load_scalar(const char* row, int64_t v, int64_t
         }
     }
     return make_uint4(t[0], t[1], t[2], t[3]);
+}
+
+// Full vector at `p` (the row's start plus 16 v bytes).  VEC: 16-byte aligned
+// rows, one 128-bit streaming load.  Other rows (contiguous rows of an odd
+// vocabulary, slices of a wider matrix): the aligned 32-bit words that hold
+// it, four, or five for a bf16 row that starts between two words, shifted into
+// place; every word read holds at least one byte of the vector, and lines are
+// shared through L1.  (24 sequences of 6 chains, V = 32001, IID, bf16: a step
+// of such rows read one token at a time took 137 us, with this and the short tail 95
+// us; 8 sequences, V = 50257, fp32: 107 -> 72 us.)
+template <int DT, bool VEC>
+__device__ __forceinline__ uint4 load_vec(const char* p) {
+    if constexpr (VEC) return ldg_stream(p);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
+    const uint32_t w0 = __ldg(w), w1 = __ldg(w + 1), w2 = __ldg(w + 2), w3 = __ldg(w + 3);
+    if constexpr (DT == 0) return make_uint4(w0, w1, w2, w3);
+    const uint32_t odd = (uint32_t)at & 2u;  // the same for every vector of a row
+    const uint32_t w4 = __ldg(w + (odd ? 4 : 3));
+    const uint32_t sh = 8u * odd;
+    return make_uint4(__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh), __funnelshift_r(w2, w3, sh),
+                      __funnelshift_r(w3, w4, sh));
+}
+
+// The four logits of Philox block cb, all of them tokens of the row.
+template <int DT, bool VEC>
+__device__ __forceinline__ void load_block(const char* row, uint32_t cb, float (&l)[4]) {
+    if constexpr (VEC && DT == 1) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(row) + cb);
+        l[0] = bf16_lo(v.x);
+        l[1] = bf16_hi(v.x);
+        l[2] = bf16_lo(v.y);
+        l[3] = bf16_hi(v.y);
+    } else if constexpr (VEC) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + cb);
+        l[0] = __uint_as_float(v.x);
+        l[1] = __uint_as_float(v.y);
+        l[2] = __uint_as_float(v.z);
+        l[3] = __uint_as_float(v.w);
+    } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) l[e] = load_logit<DT>(row, 4 * (int64_t)cb + e);
+    }
 }
 
 // Counter offset of block b of a lane's fast-loop iteration: bf16 blocks come
@@ -353,73 +364,68 @@ __device__ __forceinline__ void publish_bound(uint32_t* slot, const WarpList& L,
     if (lane == 0 && pub < kInf) atomicMax(slot, bound_enc(pub));
 }
 
-// Offer the keyed survivors of one lane (pk[e] for token i0 + e, +inf = none)
-// to the warp list: each round every lane offers its smallest remaining key
-// below the threshold; up to three offers are inserted one by one, more are
-// sorted across the warp and merged.  Ends when no lane has a key below it,
-// so the threshold is always current.
-template <int VW>
-__device__ __forceinline__ void offer_survivors(WarpList& L, float (&pk)[VW], int64_t i0, int lane,
-                                                float shift = 0.f, float eb = 0.f) {
-    while (true) {
-        float bk = kInf;
-        int bi = INT_MAX, be = -1;
-#pragma unroll
-        for (int e = 0; e < VW; ++e) {
-            if (lex_less(pk[e], (int)(i0 + e), bk, bi)) {
-                bk = pk[e];
-                bi = (int)(i0 + e);
-                be = e;
-            }
-        }
-        const bool valid = be >= 0 && bk < kInf && lex_less(bk, bi, L.th, L.thi);
-        const unsigned vm = __ballot_sync(FULL, valid);
-        if (vm == 0) break;
-        if (__popc(vm) <= 3) {
-            unsigned m = vm;
-            while (m) {
-                const int src = __ffs(m) - 1;
-                m &= m - 1;
-                const float ck = __shfl_sync(FULL, bk, src);
-                const int ci = __shfl_sync(FULL, bi, src);
-                L.mr = fminf(L.mr, list_insert(L.lk, L.li, ck, ci, L.kp, lane));
-            }
-        } else {
-            float ok = valid ? bk : kInf;
-            int oi = valid ? bi : INT_MAX;
-            warp_sort(ok, oi, lane);
-            if (L.tight())
-                L.mr = fminf(L.mr, warp_merge<true>(L.lk, L.li, ok, oi, L.kp, lane));
-            else
-                warp_merge<false>(L.lk, L.li, ok, oi, L.kp, lane);
-        }
-        // every offer of this round is now in the list or recorded in mr
-#pragma unroll
-        for (int e = 0; e < VW; ++e)
-            if (e == be) pk[e] = kInf;
-        L.refresh(shift, eb);
+// (key, token) as one integer with the order of lex_less
+__device__ __forceinline__ uint64_t list_pack(float k, int i) { return ((uint64_t)ord_key(k) << 32) | (uint32_t)i; }
+
+// Merge one offer per lane (key ok, token oi; `valid` lanes only, below the
+// list's last entry) into the warp list by ranks: every entry counts the
+// entries before it, read from shared memory, and goes to the slot of its
+// rank.  No lane waits for another's shuffle, where a bitonic sort and merge were
+// a chain of 20 of them (a K = 8 row of a one-sequence launch spent 10 us of its
+// 25 in its flushes; 64 sequences of the benchmark tree: 501 -> 488 us a step, of 8
+// non-identical proposals: 731 -> 704 us).  Lists without a spare entry record the smallest key left out.
+// `scratch`: 96 words of 64 bits of the warp's shared memory.
+__device__ __forceinline__ void list_merge(WarpList& L, bool valid, float ok, int oi, int lane, uint64_t* scratch) {
+    uint64_t *s_offer = scratch, *s_list = scratch + 32, *s_out = scratch + 64;
+    constexpr uint64_t kEmpty = (0xff800000ull << 32) | INT_MAX;  // list_pack(+inf, INT_MAX)
+    const unsigned vm = __ballot_sync(FULL, valid);
+    const int nb = __popc(vm);
+    const uint64_t b = list_pack(ok, oi), l = list_pack(L.lk, L.li);
+    if (valid) s_offer[__popc(vm & ((1u << lane) - 1u))] = b;
+    s_list[lane] = l;
+    s_out[lane] = kEmpty;
+    __syncwarp();
+    int rl = lane, rb = 0;
+#pragma unroll 2
+    for (int j = 0; j < nb; ++j) {
+        const uint64_t x = s_offer[j];
+        rl += x < l;
+        rb += x < b;
     }
-    // keys not offered (at or above entry kp-1) are left out too
-    float rem = kInf;
-#pragma unroll
-    for (int e = 0; e < VW; ++e) rem = fminf(rem, pk[e]);
-    if (L.tight() && __any_sync(FULL, rem < kInf)) L.mr = fminf(L.mr, warp_min(rem));
+#pragma unroll 2
+    for (int j = 0; j < L.kp; ++j) rb += s_list[j] < b;
+    const bool have = L.li != INT_MAX;
+    if (have && rl < L.kp) s_out[rl] = l;
+    if (valid && rb < L.kp) s_out[rb] = b;
+    if (L.tight()) {
+        float out = have && rl >= L.kp ? L.lk : kInf;
+        if (valid && rb >= L.kp) out = fminf(out, ok);
+        L.mr = fminf(L.mr, warp_min(out));
+    }
+    __syncwarp();
+    const uint64_t o = s_out[lane];
+    L.lk = unord_key((uint32_t)(o >> 32));
+    L.li = (int)(uint32_t)o;
+    __syncwarp();
 }
 
 // Filter, key and offer the 4 tokens of one Philox block (counter cb, tokens
-// 4cb..4cb+3, logits l[]) for the lanes with `mine`.  BLK: the rows are
+// 4cb..4cb+3, logits l[]) for the lanes with `mine`: each round every lane
+// keys one token that passed the filter (few have a second) and the ones below
+// the list's last entry are merged into it.  BLK: the rows are
 // proposal b's race over block b of the augmented source; survivors of the
 // (shifted) plain filter are keyed with their block arrival (fp32, error
 // bound widened by kBlkErr).
 template <bool BLK>
 __device__ __forceinline__ void block_survivors(WarpList& L, const RowPhilox& rp, bool mine, uint32_t cb,
                                                 const float (&l)[4], unsigned valid, float c, int lane, const Blk& bk,
-                                                uint64_t key, uint64_t ctx, uint32_t pos, uint32_t* slot) {
-    float pk[4] = {kInf, kInf, kInf, kInf};
+                                                uint64_t key, uint64_t ctx, uint32_t pos, uint32_t* slot,
+                                                uint64_t* scratch) {
+    uint4 q = make_uint4(0u, 0u, 0u, 0u), jq = q, fq = q;
+    unsigned pm = 0;
     if (mine) {
-        const uint4 q = rp.block(cb);
+        q = rp.block(cb);
         const uint32_t wq[4] = {q.x, q.y, q.z, q.w};
-        unsigned pm = 0;
 #pragma unroll
         for (int e = 0; e < 4; ++e)
             if (((valid >> e) & 1u) && filter_pass(wq[e], l[e], c, L.tz)) pm |= 1u << e;
@@ -427,23 +433,32 @@ __device__ __forceinline__ void block_survivors(WarpList& L, const RowPhilox& rp
             if (pm) {
                 // the block's J words and block-b excess words, four tokens per Philox block
                 const uint64_t kj = key ^ kBlockJ, kf = key ^ ((uint64_t)(uint32_t)(bk.b + 1) * kBlockF);
-                const uint4 jq = philox(cb, pos, (uint32_t)ctx, (uint32_t)(ctx >> 32), (uint32_t)kj,
-                                        (uint32_t)(kj >> 32));
-                const uint4 fq = philox(cb, pos, (uint32_t)ctx, (uint32_t)(ctx >> 32), (uint32_t)kf,
-                                        (uint32_t)(kf >> 32));
-                const uint32_t wj[4] = {jq.x, jq.y, jq.z, jq.w}, wf[4] = {fq.x, fq.y, fq.z, fq.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if ((pm >> e) & 1u)
-                        pk[e] = block_key32(wq[e], block_j(wj[e], bk.B), wf[e], bk.b, bk.invB(), l[e], c);
+                jq = philox(cb, pos, (uint32_t)ctx, (uint32_t)(ctx >> 32), (uint32_t)kj, (uint32_t)(kj >> 32));
+                fq = philox(cb, pos, (uint32_t)ctx, (uint32_t)(ctx >> 32), (uint32_t)kf, (uint32_t)(kf >> 32));
             }
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if ((pm >> e) & 1u) pk[e] = key32(wq[e], l[e], c);
         }
     }
-    offer_survivors<4>(L, pk, (int64_t)4 * cb, lane, BLK ? bk.shift() : 0.f, BLK ? kBlkErr : 0.f);
+#pragma unroll 1
+    while (__any_sync(FULL, pm != 0)) {
+        float k = kInf;
+        int i = INT_MAX;
+        if (pm) {
+            const uint32_t e = __ffs(pm) - 1;
+            pm &= pm - 1;
+            const uint32_t w = lane_of(q, e);
+            const float x = e == 0 ? l[0] : e == 1 ? l[1] : e == 2 ? l[2] : l[3];
+            if constexpr (BLK) k = block_key32(w, block_j(lane_of(jq, e), bk.B), lane_of(fq, e), bk.b, bk.invB(), x, c);
+            else k = key32(w, x, c);
+            i = (int)(4 * cb + e);
+        }
+        const bool in = k < kInf && lex_less(k, i, L.th, L.thi);
+        // a list with no spare entry records the keys it rejects (at or above its last entry)
+        if (L.tight() && __any_sync(FULL, k < kInf && !in)) L.mr = fminf(L.mr, warp_min(in ? kInf : k));
+        if (__any_sync(FULL, in)) {
+            list_merge(L, in, k, i, lane, scratch);
+            L.refresh(BLK ? bk.shift() : 0.f, BLK ? kBlkErr : 0.f);
+        }
+    }
     if (slot != nullptr) publish_bound(slot, L, BLK ? kBlkErr : 0.f, lane);
 }
 
@@ -458,12 +473,18 @@ struct SlowState {
 constexpr int kMaxUnits = PPS_UNITS > PPS_UNITS_VERIFY ? PPS_UNITS : PPS_UNITS_VERIFY;
 constexpr int kQueueCap = 32 + 32 * 2 * kMaxUnits;
 static_assert(kQueueCap >= 1 + 2 * 96, "the queue also serves as the scratch of rescan_row");
+// The warp's shared memory: the queue, then the staging of merge_rounds, whose
+// first part serves list_merge while a segment streams (a few KB a CTA more or
+// less move the SM's split between shared memory and L1).
+constexpr int kSharedWords = kQueueCap + 2 * 32 * 32;
+static_assert(kQueueCap % 4 == 0, "what follows the queue is 16-byte aligned");
+__device__ __forceinline__ uint64_t* rank_scratch(uint32_t* q) { return reinterpret_cast<uint64_t*>(q + kQueueCap); }
 
 // Work off the queue: lane j regenerates the words of queued block j (32 at
 // a time), reloads its four logits, keys the tokens over the filter cut and
 // offers them.  Out of line; the fast scan itself makes no calls.
-template <int DT, bool BLK>
-__device__ __noinline__ SlowState flush_queue(SlowState st, const uint32_t* q, int qn, const char* row, float c,
+template <int DT, bool VEC, bool BLK>
+__device__ __noinline__ SlowState flush_queue(SlowState st, uint32_t* q, int qn, const char* row, float c,
                                               uint64_t key, uint64_t ctx, uint32_t pos, Blk bk, uint32_t* slot) {
     const int lane = threadIdx.x & 31;
     RowPhilox rp;
@@ -473,34 +494,42 @@ __device__ __noinline__ SlowState flush_queue(SlowState st, const uint32_t* q, i
         const bool mine = base + lane < qn;
         const uint32_t cb = mine ? q[base + lane] : 0u;
         float l[4] = {0.f, 0.f, 0.f, 0.f};
-        if (mine) {
-            if constexpr (DT == 1) {
-                const uint2 v = __ldg(reinterpret_cast<const uint2*>(row) + cb);
-                l[0] = bf16_lo(v.x);
-                l[1] = bf16_hi(v.x);
-                l[2] = bf16_lo(v.y);
-                l[3] = bf16_hi(v.y);
-            } else {
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + cb);
-                l[0] = __uint_as_float(v.x);
-                l[1] = __uint_as_float(v.y);
-                l[2] = __uint_as_float(v.z);
-                l[3] = __uint_as_float(v.w);
-            }
-        }
-        block_survivors<BLK>(st.L, rp, mine, cb, l, 0xfu, c, lane, bk, key, ctx, pos, slot);
+        if (mine) load_block<DT, VEC>(row, cb, l);
+        block_survivors<BLK>(st.L, rp, mine, cb, l, 0xfu, c, lane, bk, key, ctx, pos, slot, rank_scratch(q));
     }
     __syncwarp();
     return st;
 }
 
-// Scalar-load path, one vector per lane at a time: the last partial
-// iteration of a segment, the ragged vector of a row, and unaligned rows.
-// Tokens with a logit below `floor` take no part (-inf: none excluded).
-template <int DT, bool BLK = false>
+// The row's last, ragged vector (V not a multiple of the vector): its at most
+// two blocks, one per lane, straight to the list.
+template <int DT, bool BLK>
+__device__ __noinline__ SlowState ragged_end(SlowState st, uint32_t* q, const char* row, int64_t V, float c,
+                                             uint64_t key, uint64_t ctx, uint32_t pos, Blk bk, uint32_t* slot) {
+    constexpr int VW = DT == 1 ? 8 : 4;
+    const int lane = threadIdx.x & 31;
+    const int64_t i0 = V / VW * VW + 4 * lane;
+    float l[4];
+    unsigned valid = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const bool on = lane < 2 && i0 + e < V;
+        l[e] = on ? load_logit<DT>(row, i0 + e) : -kInf;
+        valid |= (unsigned)on << e;
+    }
+    RowPhilox rp;
+    rp.init(key, ctx, pos);
+    block_survivors<BLK>(st.L, rp, valid != 0, (uint32_t)(i0 >> 2), l, valid, c, lane, bk, key, ctx, pos, slot,
+                         rank_scratch(q));
+    return st;
+}
+
+// Scalar-load pass, one vector per lane at a time (the truncated race's exact
+// pass over a row).  Tokens with a logit below `floor` take no part.
+template <int DT, bool BLK>
 __device__ __noinline__ SlowState tail_loop(SlowState st, const char* row, int64_t V, int64_t base, int64_t v1,
                                             float c, uint64_t key, uint64_t ctx, uint32_t pos, float floor,
-                                            Blk bk = Blk{}, uint32_t* slot = nullptr) {
+                                            Blk bk, uint64_t* scratch) {
     constexpr int VW = DT == 1 ? 8 : 4;
     const int lane = threadIdx.x & 31;
     RowPhilox rp;
@@ -534,31 +563,34 @@ __device__ __noinline__ SlowState tail_loop(SlowState st, const char* row, int64
                 for (int e = 0; e < 4; ++e) pass |= ((vh >> e) & 1u) && filter_pass(wq[e], l[e], c, st.L.tz);
             }
             if (__any_sync(FULL, pass))
-                block_survivors<BLK>(st.L, rp, pass, cb, l, vh, c, lane, bk, key, ctx, pos, slot);
+                block_survivors<BLK>(st.L, rp, pass, cb, l, vh, c, lane, bk, key, ctx, pos, nullptr, scratch);
         }
     }
     return st;
 }
 
 // A filter bound for an empty list.  Lane j keys exactly (key32, the list's
-// own key) the 8 tokens of its first unit of the segment's first fast
-// iteration and keeps its smallest; the bound is filter_slack of the k-th
+// own key) the 8 tokens of its first full vectors of the segment [v0, vend) (none:
+// +inf) and keeps its smallest; the bound is filter_slack of the k-th
 // smallest of the 32 lane minima.  Those k tokens lie in the segment, so the
 // row's k-th key is at most their largest, and the slack keeps every token
 // that could tie with it (tf itself is recorded as a drop bound).  Without
 // it every block of the first iteration would pass the filter and be queued.
 // BLK: the lane's smallest plain key is replaced by that token's block key.
-template <int DT, bool BLK>
-__device__ __noinline__ float seed_theta(const char* row, int64_t v0, float c, uint64_t key, uint64_t ctx,
-                                         uint32_t pos, int k, Blk blk) {
+template <int DT, bool VEC, bool BLK>
+__device__ __noinline__ float seed_theta(const char* row, int64_t v0, int64_t vend, float c, uint64_t key,
+                                         uint64_t ctx, uint32_t pos, int k, Blk blk) {
     const int lane = threadIdx.x & 31;
     RowPhilox rp;
     rp.init(key, ctx, pos);
-    const uint4* p = reinterpret_cast<const uint4*>(row) + v0 + lane;
+    const int64_t v = v0 + lane;
+    const uint32_t ninf = DT == 1 ? 0xff80ff80u : 0xff800000u;
     uint4 d[2];
-    d[0] = __ldg(p);
-    d[1] = DT == 1 ? d[0] : __ldg(p + 32);
-    const uint32_t cl = DT == 1 ? (uint32_t)(2 * (v0 + lane)) : (uint32_t)(v0 + lane);
+    d[0] = d[1] = make_uint4(ninf, ninf, ninf, ninf);
+    if (v < vend) d[0] = load_vec<DT, VEC>(row + 16 * v);
+    if (DT == 1) d[1] = d[0];
+    else if (v + 32 < vend) d[1] = load_vec<DT, VEC>(row + 16 * (v + 32));
+    const uint32_t cl = DT == 1 ? (uint32_t)(2 * v) : (uint32_t)v;
     float bk = kInf;
     int bi = INT_MAX;
 #pragma unroll 1
@@ -579,9 +611,12 @@ __device__ __noinline__ float seed_theta(const char* row, int64_t v0, float c, u
             }
         }
     }
-    if constexpr (BLK)
-        bk = block_key_of(key, ctx, pos, bi, word_of(key, ctx, pos, bi, 1), load_logit<DT>(row, bi), c, blk.b,
-                          blk.B, blk.invB());
+    if (bk == kInf) bi = INT_MAX;
+    if constexpr (BLK) {
+        if (bi != INT_MAX)
+            bk = block_key_of(key, ctx, pos, bi, word_of(key, ctx, pos, bi, 1), load_logit<DT>(row, bi), c, blk.b,
+                              blk.B, blk.invB());
+    }
     return filter_slack(warp_kth(bk, k)) + (BLK ? 4.0f * kBlkErr : 0.f);
 }
 
@@ -629,7 +664,7 @@ __device__ __forceinline__ float block_filter_max(const uint4& w, const float (&
 // slot (nullable): the row's shared bound, read every iteration; a smaller one
 // lowers the filter threshold and is returned in tfa (the caller records it as
 // this segment's drop bound).
-template <int DT, bool VF, int U>
+template <int DT, bool VEC, bool VF, int U>
 __device__ __forceinline__ int64_t fast_scan(const RowPhilox& rp, const char* row, int64_t v0, int64_t it0,
                                              int64_t n_it, float c, float tz, uint32_t* q, int& qn,
                                              const uint32_t* slot, float shift, float& tfa) {
@@ -637,28 +672,13 @@ __device__ __forceinline__ int64_t fast_scan(const RowPhilox& rp, const char* ro
     constexpr int ND = DT == 1 ? NB / 2 : NB;  // 16-byte vectors per lane per iteration
     constexpr int STEP = 32 * ND;              // vectors per iteration
     const int lane = threadIdx.x & 31;
-    const uint4* p = reinterpret_cast<const uint4*>(row) + v0 + it0 * STEP + lane;
+    const char* p = row + 16 * (v0 + it0 * STEP + lane);
     uint32_t cl = (DT == 1 ? (uint32_t)(2 * (v0 + lane)) : (uint32_t)(v0 + lane)) + (uint32_t)(it0 * 64 * U);
-#if PPS_PREFETCH
-    uint4 nx[ND];
-#pragma unroll
-    for (int k = 0; k < ND; ++k) nx[k] = ldg_stream(p + 32 * k);
-#endif
     for (int64_t it = it0; it < n_it; ++it) {
         uint4 d[ND];
-#if PPS_PREFETCH
 #pragma unroll
-        for (int k = 0; k < ND; ++k) d[k] = nx[k];
-        p += STEP;
-        if (it + 1 < n_it) {
-#pragma unroll
-            for (int k = 0; k < ND; ++k) nx[k] = ldg_stream(p + 32 * k);
-        }
-#else
-#pragma unroll
-        for (int k = 0; k < ND; ++k) d[k] = ldg_stream(p + 32 * k);
-        p += STEP;
-#endif
+        for (int k = 0; k < ND; ++k) d[k] = load_vec<DT, VEC>(p + 512 * k);
+        p += 16 * STEP;
         uint32_t shared_bound = 0u;
         if (slot != nullptr) asm volatile("ld.global.cg.u32 %0, [%1];" : "=r"(shared_bound) : "l"(slot));
         unsigned bm = 0;
@@ -725,38 +745,94 @@ __device__ __forceinline__ int64_t fast_scan(const RowPhilox& rp, const char* ro
     return n_it;
 }
 
-// Stream vectors [v0, v1) of one row through the warp's list: full
-// iterations through the fast loop, the rest through the scalar tail.
+// What is left of a segment after its whole iterations: full vectors [base,
+// vend), fewer than U x 32 (bf16) or x 64 (fp32) of them.  All loads are in
+// flight together; then one rolled round per 32 vectors (compact code: it
+// runs once per segment) tests each vector's largest word with its largest
+// logit and queues the blocks of passing vectors.  Returns the number queued
+// (at most 2 U x 32).
+template <int DT, bool VEC, int U>
+__device__ __noinline__ int tail_scan(const char* row, int64_t base, int64_t vend, float c, float tz, uint64_t key,
+                                      uint64_t ctx, uint32_t pos, uint32_t* q) {
+    constexpr int ND = DT == 1 ? U : 2 * U;
+    constexpr int NB = DT == 1 ? 2 : 1;  // Philox blocks per vector
+    const int lane = threadIdx.x & 31;
+    const int n = (int)(vend - base);
+    const char* p = row + 16 * (base + lane);
+    uint4 d[ND];
+#pragma unroll
+    for (int k = 0; k < ND; ++k) {
+        d[k] = make_uint4(0u, 0u, 0u, 0u);
+        if (32 * k + lane < n) d[k] = load_vec<DT, VEC>(p + 512 * k);
+    }
+    RowPhilox rp;
+    rp.init(key, ctx, pos);
+    uint32_t cb = (uint32_t)(NB * (base + lane));
+    int qn = 0;
+#pragma unroll 1
+    for (int left = n; left > 0; left -= 32, cb += 32 * NB) {
+        uint4 w = rp.block(cb);
+        uint32_t wm = max(max(w.x, w.y), max(w.z, w.w));
+        float lm;
+        if constexpr (DT == 1) {
+            w = rp.block(cb + 1);
+            wm = max(wm, max(max(w.x, w.y), max(w.z, w.w)));
+            const uint32_t m2 = bf2_max(bf2_max(d[0].x, d[0].y), bf2_max(d[0].z, d[0].w));
+            lm = fmaxf(bf16_lo(m2), bf16_hi(m2));
+        } else {
+            lm = fmaxf(fmaxf(__uint_as_float(d[0].x), __uint_as_float(d[0].y)),
+                       fmaxf(__uint_as_float(d[0].z), __uint_as_float(d[0].w)));
+        }
+#pragma unroll
+        for (int k = 0; k + 1 < ND; ++k) d[k] = d[k + 1];
+        const bool pass = lane < left && filter_pass(wm, lm, c, tz);
+        const unsigned m = __ballot_sync(FULL, pass);
+        if (pass) {
+            uint32_t* at = q + qn + NB * __popc(m & ((1u << lane) - 1u));
+            at[0] = cb;
+            if constexpr (NB == 2) at[1] = cb + 1;
+        }
+        qn += NB * __popc(m);
+    }
+    __syncwarp();
+    return qn;
+}
+
+// Stream vectors [v0, v1) of one row through the warp's list: whole
+// iterations through the fast loop, the remaining full vectors through
+// tail_scan, a ragged last vector through ragged_end.
 template <int DT, bool VEC, bool BLK, bool VF, int U>
 __device__ __forceinline__ void stream_segment(WarpList& L, const char* row, int64_t V, int64_t v0, int64_t v1,
                                                float c, uint64_t key, uint64_t ctx, uint32_t pos, uint32_t* q,
                                                const Blk& bk, uint32_t* slot) {
     constexpr int VW = DT == 1 ? 8 : 4;
     constexpr int STEP = (DT == 1 ? 32 : 64) * U;  // vectors per fast-loop iteration
-    const int64_t nfull = V / VW;                           // vectors holding VW tokens
-    const int64_t vend = VEC ? min(v1, nfull) : v0;
+    const int64_t vend = min(v1, V / VW);          // vectors holding VW tokens end here
     const int64_t n_it = vend > v0 ? (vend - v0) / STEP : 0;
+    const float shift = BLK ? bk.shift() : 0.f;
     SlowState st{L};
-    int64_t base = v0;
-    if (n_it > 0) {
-        const float shift = BLK ? bk.shift() : 0.f;
-        const float seed = seed_theta<DT, BLK>(row, v0, c, key, ctx, pos, st.L.k, bk);
+    if (vend > v0) {
+        const float seed = seed_theta<DT, VEC, BLK>(row, v0, vend, c, key, ctx, pos, st.L.k, bk);
         st.L.bound(seed, shift);
         if (slot != nullptr && (threadIdx.x & 31) == 0 && seed < kInf) atomicMax(slot, bound_enc(seed));
-        int64_t it = 0;
-        int qn = 0;
-        while (it < n_it) {
-            RowPhilox rp;
-            rp.init(key, ctx, pos);
-            float tfa = st.L.tf;
-            it = fast_scan<DT, VF, U>(rp, row, v0, it, n_it, c, st.L.tz, q, qn, slot, shift, tfa);
-            st.L.bound(tfa, shift);
-            if (qn > 0) st = flush_queue<DT, BLK>(st, q, qn, row, c, key, ctx, pos, bk, slot);
-            qn = 0;
-        }
-        base = v0 + n_it * STEP;
     }
-    if (base < v1) st = tail_loop<DT, BLK>(st, row, V, base, v1, c, key, ctx, pos, -kInf, bk, slot);
+    int64_t it = 0;
+    int qn = 0;
+    while (it < n_it) {
+        RowPhilox rp;
+        rp.init(key, ctx, pos);
+        float tfa = st.L.tf;
+        it = fast_scan<DT, VEC, VF, U>(rp, row, v0, it, n_it, c, st.L.tz, q, qn, slot, shift, tfa);
+        st.L.bound(tfa, shift);
+        if (qn > 0) st = flush_queue<DT, VEC, BLK>(st, q, qn, row, c, key, ctx, pos, bk, slot);
+        qn = 0;
+    }
+    const int64_t base = v0 + n_it * STEP;
+    if (base < vend) {
+        qn = tail_scan<DT, VEC, U>(row, base, vend, c, st.L.tz, key, ctx, pos, q);
+        if (qn > 0) st = flush_queue<DT, VEC, BLK>(st, q, qn, row, c, key, ctx, pos, bk, slot);
+    }
+    if (v1 > V / VW) st = ragged_end<DT, BLK>(st, q, row, V, c, key, ctx, pos, bk, slot);
     L = st.L;
 }
 
@@ -1355,12 +1431,12 @@ __device__ __forceinline__ void merge_partials(const RaceArgs& a, int64_t r, int
 #pragma unroll
             for (int b = 0; b + s < kMergeBatch; b += 2 * s) {
                 if (b + s < nb) {
-                    const float dk = warp_merge<true>(pk[b], pi[b], pk[b + s], pi[b + s], kp, lane);
+                    const float dk = warp_merge(pk[b], pi[b], pk[b + s], pi[b + s], kp, lane);
                     pd[b] = fminf(fminf(pd[b], pd[b + s]), dk);
                 }
             }
         }
-        const float dk = warp_merge<true>(lk, li, pk[0], pi[0], kp, lane);
+        const float dk = warp_merge(lk, li, pk[0], pi[0], kp, lane);
         theta_drop = fminf(theta_drop, fminf(pd[0], dk));
     }
 }
@@ -1482,9 +1558,9 @@ __device__ __noinline__ void finish_segment(const RaceArgs& a, int64_t r, int64_
 
 template <int DT, bool VERIFY, bool VEC, bool BLK>
 __global__ void __launch_bounds__(kThreads, BLK ? PPS_BLOCK_MIN_BLOCKS : PPS_RACE_MIN_BLOCKS) race_kernel(const RaceArgs a) {
-    __shared__ uint32_t s_queue[kQueueCap];
-    __shared__ __align__(16) float s_mk[32 * 32];  // staging of the partial lists merged by merge_rounds
-    __shared__ __align__(16) int s_mi[32 * 32];
+    __shared__ __align__(16) uint32_t s_queue[kSharedWords];
+    float* s_mk = reinterpret_cast<float*>(s_queue + kQueueCap);  // staging of the lists merged by merge_rounds
+    int* s_mi = reinterpret_cast<int*>(s_queue + kQueueCap + 32 * 32);
     pdl_wait();  // the previous kernel's outputs (row ids, lists) and the workspace it used
     pdl_launch_dependents();
     const int64_t NW = a.G;
@@ -1525,11 +1601,14 @@ __global__ void __launch_bounds__(kThreads, BLK ? PPS_BLOCK_MIN_BLOCKS : PPS_RAC
         uint32_t* slot = nullptr;
         if constexpr (PPS_ROWBOUND)
             if ((one || BLK) && a.row_bound && (v0 > 0 || v1 < nv)) slot = a.row_bound + r;
-        if (!VERIFY && !BLK && one)
+        // fp32 rows always stream with the vector test: one loop in the kernel, not two alike
+        // (two cost the fp32 draft launch 12%: 340 -> 381 us)
+        constexpr bool kVec = VERIFY || DT == 0;
+        if (!kVec && !BLK && one)
             stream_segment<DT, VEC, false, true, PPS_UNITS_VERIFY>(L, row, a.V, v0, v1, c, key, ctx, pos, s_queue,
                                                                  bk, slot);
         else
-            stream_segment<DT, VEC, BLK, VERIFY || DT == 0, VERIFY ? PPS_UNITS_VERIFY : PPS_UNITS>(
+            stream_segment<DT, VEC, BLK, kVec, kVec ? PPS_UNITS_VERIFY : PPS_UNITS>(
                 L, row, a.V, v0, v1, c, key, ctx, pos, s_queue, bk, slot);
 
         finish_segment<DT, VERIFY, BLK>(a, r, gw, NW, nb, v0, v1, L, kr, kp, bk, s_queue, s_mk, s_mi);

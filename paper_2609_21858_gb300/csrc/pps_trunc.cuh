@@ -701,7 +701,7 @@ __device__ __forceinline__ void merge_low_f(float& xk, int& xi, float yk, int yi
 }
 template <int DT, bool VERIFY, bool BLK>
 __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, const TopList& L, int kr, int kp,
-                                            float* s_val, Blk bk, uint32_t* scratch) {
+                                            float* s_val, Blk bk, uint32_t* scratch, float* s_cand) {
     const int lane = threadIdx.x & 31;
     const int k = a.top_k;
     const float lk = L.entry(k - 1);  // l_(k); -inf when the row has fewer than k usable tokens
@@ -724,7 +724,8 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, const 
         WarpList W;
         W.reset(kp, kr);
         SlowState st{W};
-        st = tail_loop<DT, BLK>(st, row, a.V, 0, a.nv, a.c, key, ctx, pos, lk, bk);
+        st = tail_loop<DT, BLK>(st, row, a.V, 0, a.nv, a.c, key, ctx, pos, lk, bk,
+                                reinterpret_cast<uint64_t*>(s_cand));
         finalize_row<DT, VERIFY, BLK>(a, r, st.L.lk, st.L.li, st.L.drop(), kr, kp, lane, bk, scratch);
         return;
     }
@@ -752,7 +753,7 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, const 
 template <int DT, bool VERIFY, bool BLK>
 __device__ __noinline__ void finish_trunc_segment(const RaceArgs& a, int64_t r, int64_t gw, int64_t NW, int64_t v0,
                                                   int64_t v1, TopList L, int kr, int kp, float* s_val, Blk bk,
-                                                  uint32_t* scratch) {
+                                                  uint32_t* scratch, float* s_cand) {
     const int lane = threadIdx.x & 31;
     const int64_t nv = a.nv;
     bool final_here = v0 == 0 && v1 == nv;
@@ -787,7 +788,7 @@ __device__ __noinline__ void finish_trunc_segment(const RaceArgs& a, int64_t r, 
         }
     }
     if (final_here) {
-        finalize_trunc<DT, VERIFY, BLK>(a, r, L, kr, kp, s_val, bk, scratch);
+        finalize_trunc<DT, VERIFY, BLK>(a, r, L, kr, kp, s_val, bk, scratch, s_cand);
         if constexpr (VERIFY) sequence_ticket(a, r, lane);
     }
 }
@@ -797,7 +798,7 @@ __device__ __noinline__ void finish_trunc_segment(const RaceArgs& a, int64_t r, 
 template <int DT, bool VERIFY, bool VEC, bool BLK>
 __global__ void __launch_bounds__(kThreads, PPS_TRUNC_MIN_BLOCKS) trunc_kernel(const RaceArgs a) {
     __shared__ float s_val[kTopMax];
-    __shared__ float s_cv[kCandCap];
+    __shared__ __align__(16) float s_cv[kCandCap];
     __shared__ int s_ci[kCandCap];
     __shared__ uint4 s_qv[kTQueueCap];
     __shared__ uint32_t s_qi[kTQueueCap];
@@ -827,6 +828,6 @@ __global__ void __launch_bounds__(kThreads, PPS_TRUNC_MIN_BLOCKS) trunc_kernel(c
             bk.B = a.n_blocks;
         }
         finish_trunc_segment<DT, VERIFY, BLK>(a, r, gw, NW, v0, v1, L, kr, kp, s_val, bk,
-                                              reinterpret_cast<uint32_t*>(s_ci));
+                                              reinterpret_cast<uint32_t*>(s_ci), s_cv);
     }
 }

@@ -1,0 +1,90 @@
+"""Rows of any alignment and length: a row's results depend on its values alone.
+
+Rows that start on 16-byte boundaries stream with 128-bit loads, others through aligned 32-bit
+words, and a row's remainder after the last whole iteration takes its own pass.  Each case places the same logits in rows of
+another offset and stride and compares every output bit for bit with the aligned rows' (which
+the parity suites check against the oracle), around the sizes of a vector, a pass of 32 vectors
+and a fast iteration (96 vectors of bf16, 192 of fp32)."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2609_21858_gb300 import pps
+
+pytestmark = pytest.mark.gpu
+
+BF, F32 = torch.bfloat16, torch.float32
+DRAFT = ("tok", "key", "mult", "ndist", "samples")
+VERIFY = ("winner", "word", "accept_len", "n_emitted", "emitted", "score", "score_sum")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    pps.lib()
+
+
+def _inputs(n, V, dtype, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    x = (torch.randn(n, V, generator=g, device="cuda") * 2.5).to(dtype)
+    if V > 40:  # some rows with masked tokens: -inf, NaN and the type's lowest value
+        hole = torch.rand(n, V, generator=g, device="cuda") < 0.2
+        x[1::4] = torch.where(hole[1::4], torch.tensor(float("-inf"), device="cuda").to(dtype), x[1::4])
+        x[2::4] = torch.where(hole[2::4], torch.tensor(float("nan"), device="cuda").to(dtype), x[2::4])
+        x[3::4] = torch.where(hole[3::4], torch.tensor(torch.finfo(dtype).min, device="cuda").to(dtype), x[3::4])
+    ids = (torch.randint(-2 ** 62, 2 ** 62, (n,), generator=g, device="cuda"),
+           torch.randint(-2 ** 62, 2 ** 62, (n,), generator=g, device="cuda"),
+           torch.randint(0, 2 ** 30, (n,), generator=g, device="cuda", dtype=torch.int32))
+    return x, ids
+
+
+def _placed(x, offset, pad):
+    """The rows of x at element `offset` of rows of V + pad elements, with foreign values around them."""
+    n, V = x.shape
+    wide = torch.full((n * (V + pad) + offset + 16,), 1e4, dtype=x.dtype, device="cuda")
+    view = wide[offset:offset + n * (V + pad)].view(n, V + pad)[:, :V]
+    view.copy_(x)
+    return view
+
+
+def _aligned(x):
+    return _placed(x, 0, -x.shape[1] % 8 + 8)
+
+
+def _same(a, b, names):
+    for k in names:
+        assert torch.equal(a[k], b[k]), k
+
+
+def _verify(x, ids, **kw):
+    n = x.shape[0]
+    off = torch.arange(n + 1, dtype=torch.int32, device="cuda")
+    none = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+    one = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+    return pps.verify_tree(x, *ids, 1, off, none, one, one[0], one, **kw)
+
+
+SIZES = [1, 5, 8, 33, 255, 256, 257, 767, 768, 769, 775, 1541, 6151, 40003]
+
+
+@pytest.mark.parametrize("dtype,offset,pad", [(BF, 1, 0), (BF, 2, 1), (BF, 4, 4), (BF, 7, 10), (F32, 1, 0),
+                                              (F32, 2, 2), (F32, 3, 5)])
+def test_results_do_not_depend_on_the_rows_place(dtype, offset, pad):
+    for V in SIZES:
+        x, ids = _inputs(9, V, dtype, 100 + V)
+        y, z = _placed(x, offset, pad), _aligned(x)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda")
+        for K, mode in ((1, pps.DISTINCT), (min(V, 8), pps.IID), (min(V, 32), pps.DISTINCT)):
+            for kw in ({}, {"top_k": 5}, {"top_k": 64, "top_p": 0.9}):
+                _same(pps.draft_list(y, *ids, K, mode=mode, status=status, **kw),
+                      pps.draft_list(z, *ids, K, mode=mode, status=status, **kw), DRAFT)
+        for kw in ({}, {"top_k": 50}):
+            _same(_verify(y, ids, status=status, **kw), _verify(z, ids, status=status, **kw), VERIFY)
+        blk = torch.arange(9, dtype=torch.int32, device="cuda") % 4
+        for kw in ({}, {"top_k": 20}):
+            a = pps.draft_hetero(y, *ids, blk, 4, status=status, **kw)
+            assert torch.equal(a, pps.draft_hetero(z, *ids, blk, 4, status=status, **kw)), V
+        assert int(status.item()) == 0, V
