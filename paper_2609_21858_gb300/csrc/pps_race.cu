@@ -1636,7 +1636,9 @@ int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk, int64_t
     const int o = resident_ctas(kOccRace + (dtype * 3 + kind) * 2 + (vec ? 1 : 0),
                                 race_fn(dtype, verify, blk && !verify, vec), kThreads);
     int64_t g = (int64_t)device_sm_count() * o;
-    int64_t by_size = (total + kMinVecsPerWarp - 1) / kMinVecsPerWarp;
+    // a warp per row at least: rows of fewer vectors one after another in a warp add up their latencies
+    // (64 sequences of 3 rows of V = 1000, fp32: 45 -> 33 us a step)
+    const int64_t by_size = max((total + kMinVecsPerWarp - 1) / kMinVecsPerWarp, n_rows);
     if (by_size < g) g = by_size;
     if (PPS_SEG_CAP > 0 && n_rows > 0 && n_rows * PPS_SEG_CAP < g) g = n_rows * PPS_SEG_CAP;
     if (n_rows > 0) {
