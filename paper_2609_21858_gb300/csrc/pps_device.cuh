@@ -92,14 +92,6 @@ __device__ __forceinline__ uint32_t word_of(uint64_t key, uint64_t ctx, uint32_t
     return lane_of(b, (uint32_t)(i & 3));
 }
 
-// word of token i (first arrival) under a key (k0, k1) that every lane of the
-// warp holds: callers pass values known warp-uniform (e.g. from
-// __reduce_or_sync), so the compiler keeps the key schedule in uniform registers
-__device__ __forceinline__ uint32_t word_of_ukey(uint32_t k0, uint32_t k1, uint64_t ctx, uint32_t pos, int64_t i) {
-    const uint4 b = philox((uint32_t)((uint64_t)i >> 2), pos, (uint32_t)ctx, (uint32_t)(ctx >> 32), k0, k1);
-    return lane_of(b, (uint32_t)(i & 3));
-}
-
 // Row-specialised Philox for the streaming loop (first arrival, fixed row).
 // Only counter word 0 (token >> 2) varies along a row, so the products of
 // the constant words in rounds 1-2 are hoisted per row: round 1 needs one

@@ -10,20 +10,27 @@ namespace pps {
 #define FULL 0xffffffffu
 
 // Detector (App. E): every warp takes a contiguous chunk of tokens and works
-// through it a group of 128 at a time; lane l loads and scores tokens
-// 4l .. 4l+3 of the group (16-byte loads when the arrays are aligned).  When
-// the whole group has one key (the tokens of one text), the Philox key
-// schedule is warp-uniform and kept in uniform registers.  Segment sums: when a
-// group lies inside the open segment (segments of a text are usually longer
-// than a group), each lane adds its four scores and one warp reduction adds
-// the group to the segment's running sum; a group that holds a segment
-// boundary is rearranged to lane-major order (shuffles) and takes a segmented
-// warp scan per 32 tokens.  The running sum is a
+// through it a group of 128 at a time; lane l loads and scores tokens 2l,
+// 2l + 1, 64 + 2l and 65 + 2l of the group (whole lines per load when the arrays are
+// aligned), the four Philox blocks round by round side by side.  When the whole group has one key
+// (the tokens of one text), the key schedule is warp-uniform and kept in
+// uniform registers.  Segment sums: the warp keeps a window of 32 segment
+// starts, one per lane, and finds a group's segments by a ballot; a group of up
+// to kSegRounds segments takes one masked warp reduction per segment, one of
+// more is rearranged to lane-major order (shuffles) and takes a segmented warp
+// scan per 32 tokens.  The running sum of the open segment is a
 // float-float pair (an exact fp32 two-sum per addition, FP64 being slow on this
 // part) and goes to the segment's fp64 slot with one atomic per segment end the
 // warp sees (plus one at the end of its chunk).
-constexpr int kScoreAhead = 4;  // iterations whose inputs a warp loads together
-
+//
+// 10^7 tuples (280 MB with the scores): about 62 us = 4.5 TB/s, 0.66 of the measured copy rate, the segment
+// pass 17 us; 10^7 tuples in texts of 128 took 96.5 us with their p-values and take 86, 6.6 10^6
+// in ragged texts of 400 tokens 130 and 90.  The kernel issues 130 instructions a tuple (40 of them the Philox
+// block) in 55% of its cycles; copying the next group's inputs to shared memory ahead (86 us),
+// five CTAs an SM of 48 registers (86 us) and sending finished sums 32 at a time (90 and 90 us before
+// the segment pass was split) changed nothing.
+constexpr int kScoreAhead = 4;  // tuples per lane of a group
+constexpr int kSegRounds = 6;
 
 // hi + lo += v, with the rounding error of hi + v kept in lo (two-sum)
 __device__ __forceinline__ void ff_add(float& hi, float& lo, float v) {
@@ -33,8 +40,40 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float v) {
     hi = s;
 }
 
+// The first-arrival words of a lane's four tuples; UNI: under one key that the
+// whole warp holds (from warp reductions, so its schedule stays in uniform registers).
+template <bool UNI>
+__device__ __forceinline__ void words4(const int32_t (&tk)[4], const uint64_t (&kk)[4], const uint64_t (&cx)[4],
+                                       const uint32_t (&ps)[4], uint32_t klo, uint32_t khi, uint32_t (&w)[4]) {
+    uint32_t x0[4], x1[4], x2[4], x3[4], k0[4], k1[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        x0[u] = (uint32_t)((uint64_t)(int64_t)tk[u] >> 2);
+        x1[u] = ps[u];
+        x2[u] = (uint32_t)cx[u];
+        x3[u] = (uint32_t)(cx[u] >> 32);
+        k0[u] = UNI ? klo : (uint32_t)kk[u];
+        k1[u] = UNI ? khi : (uint32_t)(kk[u] >> 32);
+    }
+#pragma unroll
+    for (int r = 0; r < PPS_PHILOX_ROUNDS; ++r) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            uint32_t hi0, lo0, hi1, lo1;
+            mulhilo(kPhiloxM0, x0[u], hi0, lo0);
+            mulhilo(kPhiloxM1, x2[u], hi1, lo1);
+            x0[u] = hi1 ^ x1[u] ^ (k0[u] + (uint32_t)r * kPhiloxW0);
+            x2[u] = hi0 ^ x3[u] ^ (k1[u] + (uint32_t)r * kPhiloxW1);
+            x1[u] = lo1;
+            x3[u] = lo0;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = lane_of(make_uint4(x0[u], x1[u], x2[u], x3[u]), (uint32_t)(tk[u] & 3));
+}
+
 template <bool VEC>
-__global__ void __launch_bounds__(256) wm_score_kernel(const int32_t* __restrict__ tokens,
+__global__ void __launch_bounds__(256, 4) wm_score_kernel(const int32_t* __restrict__ tokens,
                                                        const uint64_t* __restrict__ key,
                                                        const uint64_t* __restrict__ ctx,
                                                        const uint32_t* __restrict__ pos, int64_t n, int32_t n_seg,
@@ -46,115 +85,159 @@ __global__ void __launch_bounds__(256) wm_score_kernel(const int32_t* __restrict
     if (c0 >= n) return;
     const int64_t c1 = min(n, c0 + chunk);
     const bool segs = out_sum != nullptr && seg_off != nullptr;
-    // the open segment (warp-uniform): the segment of the chunk's first token (binary search, lane 0)
-    int seg = 0;
-    int64_t seg_end = LLONG_MAX;
-    if (segs) {
-        if (lane == 0) {
-            int lo = 0, hi = n_seg;  // seg_off[lo] <= c0 < seg_off[hi]
-            while (hi - lo > 1) {
-                int mid = (lo + hi) >> 1;
-                if (seg_off[mid] <= c0)
-                    lo = mid;
-                else
-                    hi = mid;
+    // the open segment (warp-uniform) and its end; win: the start of segment wb + lane
+    int seg = 0, wb = 0;
+    int64_t seg_end = LLONG_MAX, win = LLONG_MAX;
+    // open the last segment that starts at or before t (from the window on)
+    auto open_segment = [&](int64_t t) {
+        while (true) {
+            const int m = __popc(__ballot_sync(FULL, win <= t));
+            if (m < 32) {
+                seg = wb + max(m, 1) - 1;
+                seg_end = __shfl_sync(FULL, win, max(m, 1));
+                return;
             }
-            seg = lo;
+            wb += 31;
+            win = wb + lane < n_seg ? seg_off[wb + lane] : LLONG_MAX;
         }
-        seg = __shfl_sync(FULL, seg, 0);
-        seg_end = seg + 1 < n_seg ? seg_off[seg + 1] : LLONG_MAX;
+    };
+    if (segs) {
+        // 32 probes a step: seg_off[wb] <= c0 < seg_off[hi]
+        int hi = n_seg;
+        while (hi - wb > 32) {
+            const int step = (hi - wb + 31) / 32;
+            const int64_t at = (int64_t)wb + (int64_t)lane * step;
+            const int m = __popc(__ballot_sync(FULL, at < hi && seg_off[at] <= c0));
+            wb += (max(m, 1) - 1) * step;
+            hi = min(hi, wb + step);
+        }
+        win = wb + lane < n_seg ? seg_off[wb + lane] : LLONG_MAX;
+        open_segment(c0);
     }
     float chi = 0.0f, clo = 0.0f;  // running sum of the open segment
+    auto flush = [&]() {
+        if (lane == 0 && (chi != 0.0f || clo != 0.0f)) atomicAdd(out_sum + seg, (double)chi + (double)clo);
+        chi = clo = 0.0f;
+    };
     constexpr int G = 32 * kScoreAhead;
-    static_assert(kScoreAhead == 4, "a lane holds four consecutive tuples of a group");
+    static_assert(kScoreAhead == 4, "a lane holds four tuples of a group");
     for (int64_t grp = c0; grp < c1; grp += G) {
-        // lane l holds tuples grp + 4 l .. grp + 4 l + 3 (the first nloc of them exist), loaded
-        // with 16-byte loads when the arrays allow it
-        const int64_t t0 = grp + 4 * lane;
-        const int nloc = (int)max((int64_t)0, min((int64_t)4, c1 - t0));
+        // lane l holds tuples grp + 2 l, 2 l + 1, 64 + 2 l and 65 + 2 l (bits of `on`: those that
+        // exist), so that every load and store of the warp covers whole lines
+        const int64_t t0 = grp + 2 * lane;
+        const int nleft = (int)min((int64_t)G, c1 - grp);
+        const unsigned on = nleft == G ? 0xfu
+                                       : (unsigned)(2 * lane < nleft) | ((unsigned)(2 * lane + 1 < nleft) << 1) |
+                                             ((unsigned)(2 * lane + 64 < nleft) << 2) | ((unsigned)(2 * lane + 65 < nleft) << 3);
         int32_t tk[4] = {0, 0, 0, 0};
         uint64_t kk[4] = {0, 0, 0, 0}, cx[4] = {0, 0, 0, 0};
         uint32_t ps[4] = {0, 0, 0, 0};
-        if (VEC && nloc == 4) {
-            const int4 t4 = __ldg(reinterpret_cast<const int4*>(tokens + t0));
-            const uint4 p4 = __ldg(reinterpret_cast<const uint4*>(pos + t0));
+        if (VEC && nleft == G) {
+            const int2 ta = __ldg(reinterpret_cast<const int2*>(tokens + t0)), tb = __ldg(reinterpret_cast<const int2*>(tokens + t0 + 64));
+            const uint2 pa = __ldg(reinterpret_cast<const uint2*>(pos + t0)), pb = __ldg(reinterpret_cast<const uint2*>(pos + t0 + 64));
             const ulonglong2 ka = __ldg(reinterpret_cast<const ulonglong2*>(key + t0));
-            const ulonglong2 kb = __ldg(reinterpret_cast<const ulonglong2*>(key + t0 + 2));
+            const ulonglong2 kb = __ldg(reinterpret_cast<const ulonglong2*>(key + t0 + 64));
             const ulonglong2 xa = __ldg(reinterpret_cast<const ulonglong2*>(ctx + t0));
-            const ulonglong2 xb = __ldg(reinterpret_cast<const ulonglong2*>(ctx + t0 + 2));
-            tk[0] = t4.x; tk[1] = t4.y; tk[2] = t4.z; tk[3] = t4.w;
-            ps[0] = p4.x; ps[1] = p4.y; ps[2] = p4.z; ps[3] = p4.w;
+            const ulonglong2 xb = __ldg(reinterpret_cast<const ulonglong2*>(ctx + t0 + 64));
+            tk[0] = ta.x; tk[1] = ta.y; tk[2] = tb.x; tk[3] = tb.y;
+            ps[0] = pa.x; ps[1] = pa.y; ps[2] = pb.x; ps[3] = pb.y;
             kk[0] = ka.x; kk[1] = ka.y; kk[2] = kb.x; kk[3] = kb.y;
             cx[0] = xa.x; cx[1] = xa.y; cx[2] = xb.x; cx[3] = xb.y;
         } else {
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (u < nloc) {
-                    tk[u] = tokens[t0 + u];
-                    ps[u] = pos[t0 + u];
-                    kk[u] = key[t0 + u];
-                    cx[u] = ctx[t0 + u];
+                if ((on >> u) & 1u) {
+                    const int64_t t = t0 + (u & 1) + 64 * (u >> 1);
+                    tk[u] = tokens[t];
+                    ps[u] = pos[t];
+                    kk[u] = key[t];
+                    cx[u] = ctx[t];
                 }
         }
         // one key for the whole group (the tokens of one text): its schedule in uniform registers
-        bool same = true;
-#pragma unroll
-        for (int u = 1; u < 4; ++u) same &= u >= nloc || kk[u] == kk[0];
-        const uint64_t k_any = nloc > 0 ? kk[0] : 0ull;
-        const uint32_t klo = __reduce_or_sync(FULL, (uint32_t)k_any), khi = __reduce_or_sync(FULL, (uint32_t)(k_any >> 32));
-        same &= nloc == 0 || k_any == (((uint64_t)khi << 32) | klo);
-        const bool ukey = __all_sync(FULL, same);
-        float A[4];
+        const uint32_t klo = __reduce_or_sync(FULL, (uint32_t)kk[0]), khi = __reduce_or_sync(FULL, (uint32_t)(kk[0] >> 32));
+        uint32_t odd = 0;
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            A[u] = 0.0f;
-            if (u < nloc) {
-                const uint32_t w = ukey ? word_of_ukey(klo, khi, cx[u], ps[u], (int64_t)tk[u])
-                                        : word_of(kk[u], cx[u], ps[u], (int64_t)tk[u], 1);
-                A[u] = score_kind32(w, P);
-            }
+            const uint32_t d = ((uint32_t)kk[u] ^ klo) | ((uint32_t)(kk[u] >> 32) ^ khi);
+            odd |= (on >> u) & 1u ? d : 0u;
+        }
+        uint32_t w[4];
+        if (__all_sync(FULL, odd == 0u)) words4<true>(tk, kk, cx, ps, klo, khi, w);
+        else words4<false>(tk, kk, cx, ps, 0u, 0u, w);
+        float A[4];
+        if (P.kind == 0) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) A[u] = score32(w[u]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) A[u] = score_kind32(w[u], P);
+        }
+        if (nleft < G) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (!((on >> u) & 1u)) A[u] = 0.0f;
         }
         if (out_score) {
-            if (VEC && nloc == 4)
-                *reinterpret_cast<float4*>(out_score + t0) = make_float4(A[0], A[1], A[2], A[3]);
-            else
+            if (VEC && nleft == G) {
+                *reinterpret_cast<float2*>(out_score + t0) = make_float2(A[0], A[1]);
+                *reinterpret_cast<float2*>(out_score + t0 + 64) = make_float2(A[2], A[3]);
+            } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u)
-                    if (u < nloc) out_score[t0 + u] = A[u];
+                    if ((on >> u) & 1u) out_score[t0 + (u & 1) + 64 * (u >> 1)] = A[u];
+            }
         }
         if (!out_sum) continue;
-        const int64_t gend = min(grp + 32 * kScoreAhead, c1);
+        const int64_t gend = min(grp + G, c1);
         if (segs && grp >= seg_end) {
-            // the open segment ended before this group: flush it, move to the group's first segment
-            if (lane == 0 && (chi != 0.0f || clo != 0.0f)) atomicAdd(out_sum + seg, (double)chi + (double)clo);
-            chi = clo = 0.0f;
-            do {
-                ++seg;
-            } while (seg + 1 < n_seg && seg_off[seg + 1] <= grp);
-            seg_end = seg + 1 < n_seg ? seg_off[seg + 1] : LLONG_MAX;
+            // the open segment ended before this group: flush it, open the group's first segment
+            flush();
+            open_segment(grp);
         }
         if (gend <= seg_end) {
             // the whole group lies in the open segment (or there is one segment)
-            float v = A[0];
-#pragma unroll
-            for (int u = 1; u < kScoreAhead; ++u) v += A[u];
+            float v = (A[0] + A[1]) + (A[2] + A[3]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
             ff_add(chi, clo, v);
             continue;
         }
-        // a segment boundary inside the group: a segmented scan per iteration, over the
-        // lane-major layout (iteration u, lane t: tuple grp + 32 u + t, held by lane 8 u + t / 4)
+        // segments that start inside the group, as far as the window shows them
+        const unsigned inside = __ballot_sync(FULL, win > grp && win < gend);
+        if (__popc(inside) < kSegRounds && __shfl_sync(FULL, win, 31) >= gend) {
+            // one masked reduction per segment of the group
+            int64_t s0 = grp;
+            while (true) {
+                const int64_t s1 = min(seg_end, gend);
+                const int a = (int)(s0 - grp), b = (int)(s1 - grp);
+                float v = 0.0f;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int at = 2 * lane + (u & 1) + 64 * (u >> 1);
+                    v += at >= a && at < b ? A[u] : 0.0f;
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+                ff_add(chi, clo, v);
+                if (seg_end >= gend) break;  // stays open
+                s0 = seg_end;
+                flush();
+                open_segment(s0);
+            }
+            continue;
+        }
+        // many short segments: a segmented scan per iteration, over the
+        // lane-major layout (iteration u, lane t: tuple grp + 32 u + t, pair (32 u + t) / 64 of
+        // lane 16 (u mod 2) + t / 2)
         float Am[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            const int src = 8 * u + (lane >> 2);
-            const float a0 = __shfl_sync(FULL, A[0], src), a1 = __shfl_sync(FULL, A[1], src);
-            const float a2 = __shfl_sync(FULL, A[2], src), a3 = __shfl_sync(FULL, A[3], src);
-            const int e = lane & 3;
-            Am[u] = e == 0 ? a0 : e == 1 ? a1 : e == 2 ? a2 : a3;
+            const int src = 16 * (u & 1) + (lane >> 1);
+            const float a0 = __shfl_sync(FULL, A[u & 2], src), a1 = __shfl_sync(FULL, A[(u & 2) + 1], src);
+            Am[u] = lane & 1 ? a1 : a0;
         }
-#pragma unroll
+#pragma unroll 1
         for (int u = 0; u < kScoreAhead; ++u) {
             const int64_t base = grp + 32 * u;
             if (base >= c1) break;
@@ -166,7 +249,7 @@ __global__ void __launch_bounds__(256) wm_score_kernel(const int32_t* __restrict
                 while (my + 1 < n_seg && seg_off[my + 1] <= t) ++my;
             }
             // segmented inclusive scan over the lanes of each segment run
-            float v = Am[u];
+            float v = u == 0 ? Am[0] : u == 1 ? Am[1] : u == 2 ? Am[2] : Am[3];
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const float ov = __shfl_up_sync(FULL, v, o);
@@ -176,8 +259,7 @@ __global__ void __launch_bounds__(256) wm_score_kernel(const int32_t* __restrict
             // the open segment ended before this iteration's first run: flush it
             const int s0 = __shfl_sync(FULL, my, 0);
             if (s0 != seg) {
-                if (lane == 0 && (chi != 0.0f || clo != 0.0f)) atomicAdd(out_sum + seg, (double)chi + (double)clo);
-                chi = clo = 0.0f;
+                flush();
                 seg = s0;
             }
             const int nxt = __shfl_down_sync(FULL, my, 1);
@@ -200,11 +282,13 @@ __global__ void __launch_bounds__(256) wm_score_kernel(const int32_t* __restrict
                 chi = clo = 0.0f;
             }
         }
-        seg_end = seg + 1 < n_seg ? seg_off[seg + 1] : LLONG_MAX;
+        // the window from the open segment on
+        wb = seg;
+        win = wb + lane < n_seg ? seg_off[wb + lane] : LLONG_MAX;
+        seg_end = __shfl_sync(FULL, win, 1);
     }
     // the chunk's open sum (the scan path flushes its own at the chunk's end)
-    if (out_sum && lane == 0 && (chi != 0.0f || clo != 0.0f))
-        atomicAdd(out_sum + (segs ? seg : 0), (double)chi + (double)clo);
+    if (out_sum) flush();
 }
 
 // ln Gamma(x) for x >= 16 by Stirling's asymptotic series (truncation error
@@ -288,26 +372,10 @@ constexpr int64_t kSeriesF64Min = 1 << 18;
 // first-order correction for the fp32 image of S (the m-th term carries it m
 // times: with its relative error d, the exact sum is sum + d * sum_m m r_m);
 // error below 1e-6 absolute in ln p.  From kSeriesF64Min on in fp64.
-__device__ double gamma_tail_logp(int64_t M, double S) {
-    if (!(S > 0.0)) return 0.0;
-    if (M >= kSeriesF64Min) {
-        double r = 1.0, sum = 1.0;
-        if (S >= (double)M) {
-            const double inv = 1.0 / S;
-            for (int64_t j = M - 1; j > 0; --j) {
-                r *= (double)j * inv;
-                sum += r;
-                if (r < 1e-17 * sum) break;
-            }
-            return poisson_lead(M, S, false) + log(sum);
-        }
-        for (int64_t j = M + 1;; ++j) {
-            r *= S / (double)j;
-            sum += r;
-            if (r < 1e-17 * sum) break;
-        }
-        return log1p(-exp(poisson_lead(M, S, true)) * sum);
-    }
+//
+// gamma_ratios: that corrected sum (fp32 series); gamma_from: ln P from it and
+// the leading term.  The two parts do not depend on each other.
+__device__ double gamma_ratios(int64_t M, double S) {
     const float Sf = (float)S;
     float sum, wsum;
     if (S >= (double)M) {
@@ -316,16 +384,35 @@ __device__ double gamma_tail_logp(int64_t M, double S) {
         const double e = 1.0 - S * (double)inv;
         const double d = fma(e, e, e);
         poisson_ratios<true>(M, inv, sum, wsum);
-        // tot in [1, ~1e3]: its logarithm in fp32 errs by ~1e-7 absolute
-        const double tot = (double)sum + d * (double)wsum;
-        return poisson_lead(M, S, false) + (double)logf((float)tot);
+        return (double)sum + d * (double)wsum;
     }
     const double d = (S - (double)Sf) * (double)(1.0f / Sf);  // relative error of Sf (its own error ~1e-14)
     poisson_ratios<false>(M, Sf, sum, wsum);
+    return (double)sum + d * (double)wsum;
+}
+__device__ double gamma_from(int64_t M, double S, double lead, double tot) {
+    // tot in [1, ~1e3]: its logarithm in fp32 errs by ~1e-7 absolute
+    if (S >= (double)M) return lead + (double)logf((float)tot);
     // S < M: P(N >= M) <= ~1/2, so ln(1 - P(N >= M)) in fp32 errs by ~1e-7 absolute
-    const double tot = (double)sum + d * (double)wsum;
-    const double lead = poisson_lead(M, S, true);
     return (double)log1pf(-expf((float)lead) * (float)tot);
+}
+__device__ __noinline__ double gamma_tail_long(int64_t M, double S) {
+    double r = 1.0, sum = 1.0;
+    if (S >= (double)M) {
+        const double inv = 1.0 / S;
+        for (int64_t j = M - 1; j > 0; --j) {
+            r *= (double)j * inv;
+            sum += r;
+            if (r < 1e-17 * sum) break;
+        }
+        return poisson_lead(M, S, false) + log(sum);
+    }
+    for (int64_t j = M + 1;; ++j) {
+        r *= S / (double)j;
+        sum += r;
+        if (r < 1e-17 * sum) break;
+    }
+    return log1p(-exp(poisson_lead(M, S, true)) * sum);
 }
 
 // Chernoff bound on ln P(U_1 + ... + U_M >= S): the exponent
@@ -366,19 +453,43 @@ __device__ double chernoff_u_logp(int64_t M, double S) {
     return e < 0.0 ? e : 0.0;
 }
 
-// per-segment ln p-values from the segment sums (kind 0 Gamma tail, 1 Chernoff on U)
-__global__ void seg_logp_kernel(int64_t n, int32_t n_seg, const int64_t* __restrict__ seg_off,
-                                const double* __restrict__ sums, int kind, double* out_logp) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_seg) return;
-    const int64_t M = seg_off ? seg_off[g + 1] - seg_off[g] : n;
+// per-segment ln p-values from the segment sums (kind 0 Gamma tail, 1 Chernoff on U).
+// A CTA takes kLogpSegs segments; for the Gamma tail its second half of warps
+// evaluates the leading terms (a chain of fp64) while the first half runs the fp32
+// series of the same segments: each is a latency chain of about the same length
+// (one thread for both: 16400 segments of 400 tokens 111 us with their scores, now 91).
+constexpr int kLogpSegs = 64;
+__global__ void __launch_bounds__(2 * kLogpSegs) seg_logp_kernel(int64_t n, int32_t n_seg,
+                                                                  const int64_t* __restrict__ seg_off,
+                                                                  const double* __restrict__ sums, int kind,
+                                                                  double* out_logp) {
+    __shared__ double s_lead[kLogpSegs];
+    const int i = threadIdx.x % kLogpSegs;
+    const bool second = threadIdx.x >= kLogpSegs;
+    const int64_t g = (int64_t)blockIdx.x * kLogpSegs + i;
+    int64_t M = 0;
+    double S = 0.0;
+    if (g < n_seg) {
+        M = seg_off ? seg_off[g + 1] - seg_off[g] : n;
+        S = sums[g];
+    }
+    const bool series = kind == 0 && M > 0 && M < kSeriesF64Min && S > 0.0;
+    double tot = 1.0;
+    if (series) {
+        if (second) s_lead[i] = poisson_lead(M, S, !(S >= (double)M));
+        else tot = gamma_ratios(M, S);
+    }
+    __syncthreads();
+    if (second || g >= n_seg) return;
     double lp;
-    if (M <= 0)
+    if (series)
+        lp = gamma_from(M, S, s_lead[i], tot);
+    else if (M <= 0 || (kind == 0 && !(S > 0.0)))
         lp = 0.0;
     else if (kind == 0)
-        lp = gamma_tail_logp(M, sums[g]);
+        lp = gamma_tail_long(M, S);
     else if (kind == 1)
-        lp = chernoff_u_logp(M, sums[g]);
+        lp = chernoff_u_logp(M, S);
     else
         lp = __longlong_as_double(0x7ff8000000000000ll);  // NaN: no null law for this score
     out_logp[g] = lp;
@@ -636,7 +747,7 @@ cudaError_t launch_wm_score(const int32_t* tokens, const uint64_t* key, const ui
         if (e != cudaSuccess) return e;
     }
     if (out_logp && ns > 0) {
-        seg_logp_kernel<<<(ns + 127) / 128, 128, 0, stream>>>(n, ns, seg_off, out_sum, P.kind, out_logp);
+        seg_logp_kernel<<<(ns + kLogpSegs - 1) / kLogpSegs, 2 * kLogpSegs, 0, stream>>>(n, ns, seg_off, out_sum, P.kind, out_logp);
         return cudaGetLastError();
     }
     return cudaSuccess;

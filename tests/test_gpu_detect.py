@@ -139,3 +139,35 @@ def test_one_key_per_text(kind, param):
         osc, osums, _ = oracle.wm_detect(t, kk, cc, pp, sg, kind, param)
         np.testing.assert_allclose(sc.cpu().numpy(), osc, rtol=2e-5, atol=2e-6 * max(1.0, np.abs(osc).max()))
         np.testing.assert_allclose(sums.cpu().numpy(), osums, rtol=2e-5, atol=1e-4)
+
+
+# groups of 128 tuples against their segments: inside one, a few (one masked reduction each), many
+# (scan), more than a window of 32 starts at once, empty ones between; one key per segment, so groups
+# of one key and of several; array starts that allow 16-byte loads and that do not
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("lengths", [(1000, 1, 2000), (20, 30, 25, 40), (1, 2, 3), (128,) * 9, (127, 129, 128),
+                                     (600,) + (0,) * 70 + (5, 0, 0, 300), (3,) * 50 + (900,), (22, 21, 21, 21, 21, 22)])
+def test_segment_sums_at_the_edges_of_groups(lengths, shift):
+    seg = np.concatenate([[0], np.cumsum(np.tile(lengths, 5))]).astype(np.int64)
+    n = int(seg[-1])
+    tok, _, ctx, pos = _tuples(n, 7)
+    key = np.repeat(_tuples(len(seg) - 1, 8)[1], np.diff(seg))
+    def at(x):
+        wide = torch.empty(n + 8, dtype=x.dtype, device="cuda")
+        wide[shift:shift + n] = x
+        return wide[shift:shift + n]
+    k, c, p = (at(x) for x in dev_ids(key, ctx, pos))
+    sc, sums, logp = pps.wm_detect(at(torch.as_tensor(tok).cuda()), k, c, p, torch.as_tensor(seg).cuda())
+    torch.cuda.synchronize()
+    sc, sums, logp = sc.cpu().numpy(), sums.cpu().numpy(), logp.cpu().numpy()
+    osc, _, _ = oracle.wm_detect(tok, key, ctx, pos, seg, pps.SCORE_AARONSON, 0.0)
+    np.testing.assert_allclose(sc, osc, rtol=2e-5, atol=2e-6 * max(1.0, np.abs(osc).max()))
+    for g in range(len(seg) - 1):
+        x = sc[seg[g]:seg[g + 1]].astype(np.float64)
+        # a group's sum adds 2 + 5 roundings of 2^-24; the running sum is a compensated pair
+        assert abs(sums[g] - x.sum()) <= 8 * 2.0 ** -24 * x.sum(), g
+        if len(x):
+            want = oracle.gamma_tail_logp(len(x), float(sums[g]))
+            assert abs(logp[g] - want) <= logp_tol_gamma(len(x), float(sums[g]), want), g
+        else:
+            assert logp[g] == 0.0
