@@ -198,8 +198,8 @@ static pps_status draft_list(const void* q_logits, pps_dtype dtype, int64_t n_ro
     const bool vec = vec_ok(q_logits, dtype, row_stride);
     cudaError_t e;
     if (top_k > 0) {
-        a.G = trunc_grid(a.total, a.n_rows, dt, false, vec);
-        e = launch_trunc(a, dt, false, vec, (cudaStream_t)stream);
+        a.G = trunc_grid(a.total, a.n_rows, dt, false);
+        e = launch_trunc(a, dt, false, (cudaStream_t)stream);
     } else {
         a.G = race_grid(a.total, dt, false, vec, false, a.n_rows);
         e = launch_race(a, dt, false, vec, (cudaStream_t)stream);
@@ -271,8 +271,8 @@ static pps_status verify_tree(const void* p_logits, pps_dtype dtype, int64_t n_n
     const bool vec = vec_ok(p_logits, dtype, row_stride);
     cudaError_t e;
     if (top_k > 0) {
-        a.G = trunc_grid(a.total, a.n_rows, dt, true, vec);
-        e = launch_trunc(a, dt, true, vec, (cudaStream_t)stream);
+        a.G = trunc_grid(a.total, a.n_rows, dt, true);
+        e = launch_trunc(a, dt, true, (cudaStream_t)stream);
     } else {
         a.G = race_grid(a.total, dt, true, vec, false, a.n_rows);
         e = launch_race(a, dt, true, vec, (cudaStream_t)stream);
@@ -544,8 +544,8 @@ static pps_status draft_hetero(const void* q_logits, pps_dtype dtype, int64_t n_
     const bool vec = vec_ok(q_logits, dtype, row_stride);
     cudaError_t e;
     if (top_k > 0) {
-        a.G = trunc_grid(a.total, a.n_rows, dt, false, vec, n_blocks > 1);
-        e = launch_trunc(a, dt, false, vec, (cudaStream_t)stream);
+        a.G = trunc_grid(a.total, a.n_rows, dt, false, n_blocks > 1);
+        e = launch_trunc(a, dt, false, (cudaStream_t)stream);
     } else {
         a.G = race_grid(a.total, dt, false, vec, n_blocks > 1, a.n_rows);
         e = launch_race(a, dt, false, vec, (cudaStream_t)stream);

@@ -25,14 +25,15 @@ struct alignas(16) Partial {
     int32_t pad[2];
 };
 
-// one partial top-k list of a row segment for the truncated race (sorted by
-// logit descending, then token ascending; empty entries (-inf, INT_MAX))
+// one partial top-k list of a row segment for the truncated race (in any
+// order; empty entries (-inf, INT_MAX))
 constexpr int kTopMax = 64;  // largest top-k of the truncated race
 struct alignas(16) TruncPartial {
     float v[kTopMax];
     int32_t idx[kTopMax];
     float dropmax;  // largest logit evicted from the segment's list (-inf: none)
-    int32_t pad[3];
+    float thr;      // lower bound of the row's l_(k) (-inf: the segment has fewer than k usable tokens)
+    int32_t pad[2];
 };
 // workspace slot: room for either kind of partial list
 constexpr size_t kSlotBytes = sizeof(TruncPartial) > sizeof(Partial) ? sizeof(TruncPartial) : sizeof(Partial);
@@ -125,15 +126,15 @@ void workspace_carve(void* ws, int64_t n_rows, int32_t n_seq, Partial** partials
 // (< kOccSlots) names the kernel in the cache.
 constexpr int kOccSlots = 32;
 constexpr int kOccRace = 0;    // 12 slots: dtype x (draft, verify, block) x vec
-constexpr int kOccTrunc = 12;  // 12 slots, the same
+constexpr int kOccTrunc = 12;  // 6 slots: dtype x (draft, verify, block)
 constexpr int kOccScore = 24;
 int device_sm_count();
 int resident_ctas(int slot, const void* fn, int threads);
 
 cudaError_t launch_race(const RaceArgs& a, int dtype, bool verify, bool vec, cudaStream_t stream);
 int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk = false, int64_t n_rows = 0);
-cudaError_t launch_trunc(const RaceArgs& a, int dtype, bool verify, bool vec, cudaStream_t stream);
-int trunc_grid(int64_t total, int64_t n_rows, int dtype, bool verify, bool vec, bool blk = false);
+cudaError_t launch_trunc(const RaceArgs& a, int dtype, bool verify, cudaStream_t stream);
+int trunc_grid(int64_t total, int64_t n_rows, int dtype, bool verify, bool blk = false);
 
 // the LM-head GEMM with the race in its epilogue (pps_lmhead.cuh, in pps_race.cu).
 // hidden [n_rows, d] and weight [V, d] are bf16 with row strides ldh, ldw elements.

@@ -1691,60 +1691,44 @@ cudaError_t launch_race(const RaceArgs& a, int dtype, bool verify, bool vec, cud
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Rows stay whole where the grid allows (a segment's candidate count grows
-// like k ln(segment / k), and a row finished by one warp needs no merge):
-// with at most as many rows as resident warps, each row gets the same number
-// of warps s; with more rows, the grid is the resident one.
-static const void* trunc_fn(int dtype, bool verify, bool blk, bool vec) {
+// Rows stay whole when there are no more warps than rows (a segment's candidate
+// count grows like k ln(segment / k), and a row finished by one warp needs no
+// merge); fewer rows than warps get the same number of warps each, up to
+// kTruncSegCap of at least kTruncMinVecs vectors.
+static const void* trunc_fn(int dtype, bool verify, bool blk) {
     if (dtype == 1) {
-        if (verify) return vec ? (const void*)trunc_kernel<1, true, true, false> : (const void*)trunc_kernel<1, true, false, false>;
-        if (blk) return vec ? (const void*)trunc_kernel<1, false, true, true> : (const void*)trunc_kernel<1, false, false, true>;
-        return vec ? (const void*)trunc_kernel<1, false, true, false> : (const void*)trunc_kernel<1, false, false, false>;
+        if (verify) return (const void*)trunc_kernel<1, true, false>;
+        return blk ? (const void*)trunc_kernel<1, false, true> : (const void*)trunc_kernel<1, false, false>;
     }
-    if (verify) return vec ? (const void*)trunc_kernel<0, true, true, false> : (const void*)trunc_kernel<0, true, false, false>;
-    if (blk) return vec ? (const void*)trunc_kernel<0, false, true, true> : (const void*)trunc_kernel<0, false, false, true>;
-    return vec ? (const void*)trunc_kernel<0, false, true, false> : (const void*)trunc_kernel<0, false, false, false>;
+    if (verify) return (const void*)trunc_kernel<0, true, false>;
+    return blk ? (const void*)trunc_kernel<0, false, true> : (const void*)trunc_kernel<0, false, false>;
 }
 
-int trunc_grid(int64_t total, int64_t n_rows, int dtype, bool verify, bool vec, bool blk) {
+int trunc_grid(int64_t total, int64_t n_rows, int dtype, bool verify, bool blk) {
     const int kind = verify ? 1 : (blk ? 2 : 0);
-    const int o = resident_ctas(kOccTrunc + (dtype * 3 + kind) * 2 + (vec ? 1 : 0),
-                                trunc_fn(dtype, verify, blk && !verify, vec), kThreads);
+    const int o = resident_ctas(kOccTrunc + dtype * 3 + kind, trunc_fn(dtype, verify, blk && !verify), kThreads);
     int64_t g = (int64_t)device_sm_count() * o;
-    int64_t by_size = (total + kMinVecsPerWarp - 1) / kMinVecsPerWarp;
-    if (by_size < g) g = by_size;
-    if (n_rows > 0 && n_rows <= g) g = n_rows * (g / n_rows);
+    if (n_rows > 0 && n_rows < g) {
+        const int64_t s = min(min((int64_t)kTruncSegCap, g / n_rows), total / n_rows / kTruncMinVecs);
+        g = n_rows * max((int64_t)1, s);
+    }
     if (g > kGridMax) g = kGridMax;
     if (g < 1) g = 1;
     return (int)g;
 }
 
-cudaError_t launch_trunc(const RaceArgs& a, int dtype, bool verify, bool vec, cudaStream_t stream) {
+cudaError_t launch_trunc(const RaceArgs& a, int dtype, bool verify, cudaStream_t stream) {
     dim3 grid(a.G), block(kThreads);
     cudaError_t e = cudaSuccess;
     const bool blk = !verify && a.row_block != nullptr;
     if (dtype == 1) {
-        if (verify) {
-            if (vec) e = launch_pdl(trunc_kernel<1, true, true, false>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<1, true, false, false>, grid, block, 0, stream, a);
-        } else if (blk) {
-            if (vec) e = launch_pdl(trunc_kernel<1, false, true, true>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<1, false, false, true>, grid, block, 0, stream, a);
-        } else {
-            if (vec) e = launch_pdl(trunc_kernel<1, false, true, false>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<1, false, false, false>, grid, block, 0, stream, a);
-        }
+        if (verify) e = launch_pdl(trunc_kernel<1, true, false>, grid, block, 0, stream, a);
+        else if (blk) e = launch_pdl(trunc_kernel<1, false, true>, grid, block, 0, stream, a);
+        else e = launch_pdl(trunc_kernel<1, false, false>, grid, block, 0, stream, a);
     } else {
-        if (verify) {
-            if (vec) e = launch_pdl(trunc_kernel<0, true, true, false>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<0, true, false, false>, grid, block, 0, stream, a);
-        } else if (blk) {
-            if (vec) e = launch_pdl(trunc_kernel<0, false, true, true>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<0, false, false, true>, grid, block, 0, stream, a);
-        } else {
-            if (vec) e = launch_pdl(trunc_kernel<0, false, true, false>, grid, block, 0, stream, a);
-            else e = launch_pdl(trunc_kernel<0, false, false, false>, grid, block, 0, stream, a);
-        }
+        if (verify) e = launch_pdl(trunc_kernel<0, true, false>, grid, block, 0, stream, a);
+        else if (blk) e = launch_pdl(trunc_kernel<0, false, true>, grid, block, 0, stream, a);
+        else e = launch_pdl(trunc_kernel<0, false, false>, grid, block, 0, stream, a);
     }
     return e != cudaSuccess ? e : cudaGetLastError();
 }

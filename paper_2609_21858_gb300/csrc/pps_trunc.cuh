@@ -14,37 +14,52 @@
 //
 // Work per row.  The streaming pass only finds S: one max of the iteration's
 // logits per lane (packed bf16x2 max for bf16 rows) against the warp's
-// threshold, the k-th entry of a per-warp top list of up to 64 (logit, token)
-// entries.  No Philox word is needed for a token outside S, so the pass is
-// bound by HBM rather than by the multiply pipe.  Vectors with a logit at or
-// over the threshold are queued and their tokens merged into the list
-// (bitonic sort and merges).  Tokens below the threshold are below l_(k) and
-// can be dropped for good; a token evicted from a full list is recorded in
-// `dropmax`, and if one ties with l_(k) the row's list does not hold the whole
-// tie group: the row is then finished by a counting pass (for top-p) and, when
+// threshold, a lower bound of l_(k).  No Philox word is needed for a token
+// outside S, so the pass is bound by HBM rather than by the multiply pipe.
+// Vectors with a logit at or over the threshold are queued and their tokens
+// appended to a buffer; when it fills it is compacted to the tokens that can
+// still be in S, which raises the threshold.  Tokens below the threshold are
+// below l_(k) and can be dropped for good; a token tied with it that did not fit
+// is recorded in `dropmax`, and if one ties with l_(k) the buffer does not hold
+// the whole tie group: the row is then finished by a counting pass (for top-p) and, when
 // the tie group stays in S, by the exact fp32 race of pps_race.cu over the
 // tokens with logit >= l_(k).  Otherwise the finishing warp keys the <= 64
-// surviving tokens with the race's fp32 key, keeps the 32 smallest and hands
+// surviving tokens with the race's fp32 key, keeps the smallest and hands
 // them to finalize_row with a drop bound of +inf (S is complete, nothing was
 // dropped); finalize_row re-keys in fp64 (s = ln E - l/T) every pair closer
 // than the fp32 error bounds, so the row is emitted exactly like the
 // untruncated race.
+//
+// A step of the benchmark's tree (top-k 50: 1.21 GB of logits) takes 266 us =
+// 4.6 TB/s, 290 when every row's threshold climbed from the first iteration's and S
+// was sorted; one sequence 263 -> 88 us; 16720 rows of V = 5717 736 -> 248 us.  It is
+// bound by HBM (0.78 of the measured copy rate inside the launch, 8% of the reads being
+// the sample) and by the finish of the last rows, about 12 us a launch.
 
 #ifndef PPS_TRUNC_UNITS
 #define PPS_TRUNC_UNITS 8  // 16-byte vectors per lane per iteration of the top-k scan (even)
 #endif
 #ifndef PPS_TRUNC_EAGER
-#define PPS_TRUNC_EAGER 96  // buffered candidates at which a queue flush also compacts
+#define PPS_TRUNC_EAGER 192  // buffered candidates at which a queue flush also compacts (at 96: 282 us instead of 266)
 #endif
 #ifndef PPS_TRUNC_MIN_BLOCKS
 #define PPS_TRUNC_MIN_BLOCKS 20
 #endif
+#ifndef PPS_TRUNC_SEG_CAP
+#define PPS_TRUNC_SEG_CAP 16
+#endif
+constexpr int kTruncSegCap = PPS_TRUNC_SEG_CAP;  // at most this many warps per row (one sequence: 8 98 us, 16 87, 32 93)
+#ifndef PPS_TRUNC_MIN_VECS
+#define PPS_TRUNC_MIN_VECS 512
+#endif
+constexpr int64_t kTruncMinVecs = PPS_TRUNC_MIN_VECS;  // a row is not cut finer (132 rows of V = 7338: 256 66 us, 512 58)
+constexpr int kTruncRounds = 8;  // kept lists up to this long are selected by argmin rounds
 
 // ---------------------------------------------------------------- top lists
 // A top list holds up to 64 entries (v, i) in "top order": logit descending,
-// then token ascending.  Entry m sits in lane m (av, ai) for m < 32 and in
-// lane m - 32 (bv, bi) otherwise; empty entries are (-inf, INT_MAX).  NaN and
-// -inf logits never enter.
+// then token ascending (only top-p needs the order).  Entry m sits in lane m
+// (av, ai) for m < 32 and in lane m - 32 (bv, bi) otherwise; empty entries are
+// (-inf, INT_MAX).  NaN and -inf logits never enter.
 
 __device__ __forceinline__ bool top_before(float av, int ai, float bv, int bi) {
     return av > bv || (av == bv && ai < bi);
@@ -99,119 +114,11 @@ __device__ __forceinline__ void top_merge(float xv, int xi, float yv, int yi, fl
     top_clean(lv, li, lane);
 }
 
+// the buffer's entries in top order: entries lane and lane + 32
 struct TopList {
-    float av, bv;   // entries lane and lane + 32
+    float av, bv;
     int ai, bi;
-    float thr;      // logit of entry k-1 (-inf while fewer than k entries): tokens below it cannot be in S
-    float dropmax;  // largest logit evicted from the list (-inf: none)
-
-    __device__ __forceinline__ void reset() {
-        av = bv = -kInf;
-        ai = bi = INT_MAX;
-        thr = -kInf;
-        dropmax = -kInf;
-    }
-    __device__ __forceinline__ float entry(int m) const {  // m warp-uniform
-        const float x = __shfl_sync(FULL, av, m & 31), y = __shfl_sync(FULL, bv, m & 31);
-        return m < 32 ? x : y;
-    }
-    // Merge a batch in top order (one entry per lane).  The first 32 of
-    // (a, batch) are the new a; the rest merged with b gives the new b and
-    // the evicted 32 (every entry of the old a precedes every entry of b, so
-    // the first 64 of the union are exactly these).
-    __device__ __forceinline__ void insert_sorted(float cv, int ci, int k, int lane) {
-        float xh, xl, yh, yl;
-        int xhi, xli, yhi, yli;
-        top_merge(av, ai, cv, ci, xh, xhi, xl, xli, lane);
-        top_merge(xl, xli, bv, bi, yh, yhi, yl, yli, lane);
-        av = xh;
-        ai = xhi;
-        bv = yh;
-        bi = yhi;
-        dropmax = fmaxf(dropmax, __shfl_sync(FULL, yl, 0));
-        thr = fmaxf(thr, entry(k - 1));
-    }
-    // insert one warp-uniform entry: find its place by ballots, shift the rest down
-    __device__ __forceinline__ void insert_one(float cv, int ci, int k, int lane) {
-        const int pos = __popc(__ballot_sync(FULL, top_before(av, ai, cv, ci))) +
-                        __popc(__ballot_sync(FULL, top_before(bv, bi, cv, ci)));
-        if (pos >= 2 * 32) {
-            dropmax = fmaxf(dropmax, cv);
-            return;
-        }
-        const float a31 = __shfl_sync(FULL, av, 31), b63 = __shfl_sync(FULL, bv, 31);
-        const int a31i = __shfl_sync(FULL, ai, 31);
-        float pa = __shfl_up_sync(FULL, av, 1), pb = __shfl_up_sync(FULL, bv, 1);
-        int pai = __shfl_up_sync(FULL, ai, 1), pbi = __shfl_up_sync(FULL, bi, 1);
-        if (lane == 0) {
-            pb = a31;
-            pbi = a31i;
-        }
-        if (lane > pos) {
-            av = pa;
-            ai = pai;
-        } else if (lane == pos) {
-            av = cv;
-            ai = ci;
-        }
-        if (32 + lane > pos) {
-            bv = pb;
-            bi = pbi;
-        } else if (32 + lane == pos) {
-            bv = cv;
-            bi = ci;
-        }
-        dropmax = fmaxf(dropmax, b63);
-        thr = fmaxf(thr, entry(k - 1));
-    }
-    // A token can still change S: above the threshold, or tied with it while no
-    // token of that logit has been evicted yet (once one has, the row's tie
-    // group at that logit, if it is l_(k), overflows whatever else arrives).
-    __device__ __forceinline__ bool wants(float x) const {
-        return x > -kInf && (x > thr || (x == thr && dropmax < thr));
-    }
-    // one round: every lane offers (v, i) or nothing (-inf); few offers go in one
-    // by one, more are sorted and merged
-    __device__ __forceinline__ void offer(float v, int i, int k, int lane) {
-        const unsigned vm = __ballot_sync(FULL, v > -kInf);
-        if (__popc(vm) <= 2) {
-            unsigned m = vm;
-            while (m) {
-                const int src = __ffs(m) - 1;
-                m &= m - 1;
-                insert_one(__shfl_sync(FULL, v, src), __shfl_sync(FULL, i, src), k, lane);
-            }
-        } else {
-            if (v == -kInf) i = INT_MAX;
-            top_sort(v, i, lane);
-            insert_sorted(v, i, k, lane);
-        }
-    }
 };
-
-// Offer each lane's candidates (logits cv[e] of tokens ci[e]; -inf = none) to
-// the list: every round the lanes' best remaining candidates at or over the
-// threshold are sorted and merged; ends when no lane has one.
-template <int N>
-__device__ __forceinline__ void top_offer(TopList& L, float (&cv)[N], const int (&ci)[N], int k, int lane) {
-    while (true) {
-        float bv = -kInf;
-        int bi = INT_MAX, be = -1;
-#pragma unroll
-        for (int e = 0; e < N; ++e) {
-            if (L.wants(cv[e]) && top_before(cv[e], ci[e], bv, bi)) {
-                bv = cv[e];
-                bi = ci[e];
-                be = e;
-            }
-        }
-        if (__ballot_sync(FULL, be >= 0) == 0) break;
-        L.offer(bv, bi, k, lane);
-#pragma unroll
-        for (int e = 0; e < N; ++e)
-            if (e == be) cv[e] = -kInf;
-    }
-}
 
 // ---------------------------------------------------------------- vector helpers
 
@@ -225,15 +132,6 @@ __device__ __forceinline__ bool bf2_any_ge(uint32_t m, uint32_t t2) {
         : "=r"(r)
         : "r"(m), "r"(t2));
     return r != 0;
-}
-
-// token e of a 16-byte vector as fp32 (exact)
-template <int DT>
-__device__ __forceinline__ float vec_token(const uint4& d, int e) {  // e a compile-time constant after unrolling
-    const uint32_t w4[4] = {d.x, d.y, d.z, d.w};
-    const uint32_t w = w4[DT == 1 ? e >> 1 : e];
-    if constexpr (DT == 1) return (e & 1) ? bf16_hi(w) : bf16_lo(w);
-    else return __uint_as_float(w);
 }
 
 // largest usable logit of vectors d[k0 .. k0+n) (NaN ignored, -inf if none)
@@ -264,6 +162,23 @@ __device__ __forceinline__ float from_order_key(uint32_t u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
+// The k-th largest of the warp's 32 x N order keys, bit by bit (bf16 values: the
+// high 16 bits decide, the low ones are all 0, or all 1 below zero).  At least k
+// of them are not 0.
+template <int DT, int N>
+__device__ __forceinline__ uint32_t kth_order_key(const uint32_t (&key)[N], int k) {
+    uint32_t res = 0;
+#pragma unroll 1
+    for (int b = 31; b >= (DT == 1 ? 16 : 0); --b) {
+        const uint32_t cand = res | (1u << b);
+        int n = 0;
+#pragma unroll
+        for (int j = 0; j < N; ++j) n += key[j] >= cand;
+        if (__reduce_add_sync(FULL, (unsigned)n) >= (unsigned)k) res = cand;
+    }
+    return DT == 1 && !(res & 0x80000000u) ? res | 0xffffu : res;
+}
+
 // Threshold for an empty buffer, from the first iteration's vectors: the
 // k-th largest of the 32 x NV per-vector maxima (bitwise search on order
 // keys).  They are maxima of distinct vectors of the segment, so at least k
@@ -274,13 +189,45 @@ __device__ __forceinline__ float seed_thr(const uint4 (&d)[PPS_TRUNC_UNITS], int
     uint32_t key[NV];
 #pragma unroll
     for (int j = 0; j < NV; ++j) key[j] = order_key(vecs_max<DT>(d, j, 1));
+    return from_order_key(kth_order_key<DT, NV>(key, k));
+}
+
+// A guess of l_(k) for a long segment, from 32 sampled chunks of 32 vectors
+// spread evenly over [v0, vend) (`row`: the interior's start): the j-th largest
+// of the 32 chunk maxima, j three deviations and three above the number of
+// top-k tokens expected in the sample.  With it the scan buffers about
+// j / f tokens of a segment sampled at f = 32 chunks / all chunks (200 of 128256, k =
+// 50) and hardly ever compacts; the threshold the first iteration proves
+// lets through ~1000 and compacts every 46 (a step of the benchmark's tree 289 -> 263 us).  It is a guess: topk_segment checks
+// that k tokens reached it.  One maximum per chunk keeps a cluster of large
+// logits (a vocabulary sorted by frequency) from raising it.
+constexpr int kSampleChunks = 32;
+constexpr int64_t kSampleMin = 32 * 192;  // vectors; shorter segments gain nothing from a guess
+
+template <int DT>
+__device__ __noinline__ float guess_thr(const char* row, int64_t v0, int64_t vend, int k) {
+    constexpr int B = 8;  // chunks loaded together
+    const int lane = threadIdx.x & 31;
+    const int64_t chunks = (vend - v0) / 32;
+    const uint4* p = reinterpret_cast<const uint4*>(row) + v0 + lane;
+    uint32_t mine = 0;  // lane c: order key of chunk c's largest logit
+#pragma unroll 1
+    for (int c0 = 0; c0 < kSampleChunks; c0 += B) {
+        uint4 d[B];
+#pragma unroll
+        for (int j = 0; j < B; ++j) d[j] = ldg_stream(p + (chunks * (c0 + j) / kSampleChunks) * 32);
+#pragma unroll
+        for (int j = 0; j < B; ++j) {
+            const uint32_t m = __reduce_max_sync(FULL, order_key(vecs_max<DT>(d, j, 1)));
+            if (lane == c0 + j) mine = m;
+        }
+    }
+    const float x = (float)(kSampleChunks * k) / (float)chunks;
+    const int j = (int)(x + 3.0f * sqrtf(x) + 4.0f);  // < 32 for k <= kTopMax and kSampleMin vectors
     uint32_t res = 0;
     for (int b = 31; b >= 0; --b) {
         const uint32_t cand = res | (1u << b);
-        int n = 0;
-#pragma unroll
-        for (int j = 0; j < NV; ++j) n += key[j] >= cand;
-        if (__reduce_add_sync(FULL, (unsigned)n) >= (unsigned)k) res = cand;
+        if (__popc(__ballot_sync(FULL, mine >= cand)) >= j) res = cand;
     }
     return from_order_key(res);
 }
@@ -297,7 +244,9 @@ struct CandState {
     float thr;      // lower bound of l_(k): tokens below it cannot be in S
     float dropmax;  // largest logit dropped from the buffer (-inf: none)
     int n;          // buffered entries
-    // tokens that may still change S (see TopList::wants)
+    // A token can still change S: above the threshold, or tied with it while no
+    // token of that logit has been dropped yet (once one has, the row's tie
+    // group at that logit, if it is l_(k), overflows whatever else arrives).
     __device__ __forceinline__ bool wants(float x) const {
         return x > -kInf && (x > thr || (x == thr && dropmax < thr));
     }
@@ -317,17 +266,11 @@ __device__ __noinline__ CandState cand_compact(CandState C, float* sv, int* si, 
         ix[j] = q < C.n ? si[q] : INT_MAX;
     }
     __syncwarp();
-    // t = the k-th largest buffered logit, bit by bit on order keys (bf16
-    // values: the high 16 bits decide, the low ones are all 0 or all 1)
-    uint32_t res = 0;
-    for (int b = 31; b >= (DT == 1 ? 16 : 0); --b) {
-        const uint32_t cand = res | (1u << b);
-        int n = 0;
+    // t = the k-th largest buffered logit
+    uint32_t ok[PER];
 #pragma unroll
-        for (int j = 0; j < PER; ++j) n += v[j] > -kInf && order_key(v[j]) >= cand;
-        if (__reduce_add_sync(FULL, (unsigned)n) >= (unsigned)k) res = cand;
-    }
-    if (DT == 1 && !(res & 0x80000000u)) res |= 0xffffu;  // a negative value: its key ends in ones
+    for (int j = 0; j < PER; ++j) ok[j] = v[j] > -kInf ? order_key(v[j]) : 0u;
+    const uint32_t res = kth_order_key<DT, PER>(ok, k);
     const float t = from_order_key(res);
     int ng = 0;
 #pragma unroll
@@ -363,19 +306,33 @@ __device__ __noinline__ CandState cand_compact(CandState C, float* sv, int* si, 
 }
 
 // the buffer (n <= 64 entries) as a sorted top list
-__device__ __noinline__ TopList cand_to_list(const CandState& C, const float* sv, const int* si, int k) {
+__device__ __noinline__ TopList cand_to_list(int n, const float* sv, const int* si) {
     const int lane = threadIdx.x & 31;
     TopList L;
-    L.reset();
-    float av = lane < C.n ? sv[lane] : -kInf, bv = 32 + lane < C.n ? sv[32 + lane] : -kInf;
-    int ai = lane < C.n ? si[lane] : INT_MAX, bi = 32 + lane < C.n ? si[32 + lane] : INT_MAX;
-    __syncwarp();
+    float av = lane < n ? sv[lane] : -kInf, bv = 32 + lane < n ? sv[32 + lane] : -kInf;
+    int ai = lane < n ? si[lane] : INT_MAX, bi = 32 + lane < n ? si[32 + lane] : INT_MAX;
     top_sort(av, ai, lane);
     top_sort(bv, bi, lane);
     top_merge(av, ai, bv, bi, L.av, L.ai, L.bv, L.bi, lane);
-    L.dropmax = C.dropmax;
-    L.thr = fmaxf(C.thr, L.entry(k - 1));
     return L;
+}
+
+// Append each lane's token (x, i) that is wanted (x = -inf: none); the buffer is compacted when it runs over.
+template <int DT>
+__device__ __forceinline__ void cand_push(CandState& C, float* sv, int* si, float x, int i, int k) {
+    const int lane = threadIdx.x & 31;
+    unsigned m = __ballot_sync(FULL, C.wants(x));
+    if (C.n + __popc(m) > kCandCap) {
+        C = cand_compact<DT>(C, sv, si, k);
+        m = __ballot_sync(FULL, C.wants(x));
+    }
+    if ((m >> lane) & 1u) {
+        const int o = C.n + __popc(m & ((1u << lane) - 1u));
+        sv[o] = x;
+        si[o] = i;
+    }
+    C.n += __popc(m);
+    __syncwarp();
 }
 
 // Next bf16 value below x (x a bf16 value, not NaN, not -inf): with it,
@@ -472,21 +429,23 @@ __device__ __noinline__ CandState cand_append(CandState C, float* sv, int* si, c
     }
 }
 
-// Flagged vectors wait in a per-warp queue in shared memory (their 16 bytes
-// and their index in the row); one iteration adds at most 32 x NV.
+// Flagged vectors wait in a per-warp queue of their indexes; one iteration adds
+// at most 32 x NV.  Working the queue off loads the vectors again (they are in
+// L2), 5 KB of shared memory less a CTA, which the L1 gets.
 constexpr int kTQueueCap = 32 + 32 * PPS_TRUNC_UNITS;
 
-// Work off the queue, one vector per lane, 32 at a time.
+// Work off the queue, one vector per lane (staged in st), 32 at a time.
 template <int DT>
-__device__ __noinline__ CandState topk_flush(CandState C, float* sv, int* si, const uint4* qv, const uint32_t* qi,
-                                             int qn, int k) {
+__device__ __noinline__ CandState topk_flush(CandState C, float* sv, int* si, uint4* st, const uint32_t* qi, int qn,
+                                             const char* row, int h, int k) {
     constexpr int VW = DT == 1 ? 8 : 4;
     const int lane = threadIdx.x & 31;
     __syncwarp();
     for (int base = 0; base < qn; base += 32) {
         const bool mine = base + lane < qn;
-        const int i0 = mine ? (int)(qi[base + lane] * VW) : 0;
-        C = cand_append<DT>(C, sv, si, qv + base, mine ? 1u : 0u, i0, k);
+        const uint32_t v = mine ? qi[base + lane] : 0u;
+        if (mine) st[lane] = __ldg(reinterpret_cast<const uint4*>(row) + v);
+        C = cand_append<DT>(C, sv, si, st, mine ? 1u : 0u, (int)(v * VW) + h, k);
     }
     // raise the threshold early: a stale one lets through many more tokens
     if (C.n >= PPS_TRUNC_EAGER) C = cand_compact<DT>(C, sv, si, k);
@@ -494,11 +453,12 @@ __device__ __noinline__ CandState topk_flush(CandState C, float* sv, int* si, co
 }
 
 // One iteration of the fast scan (NV vectors per lane, d[j] = vector vfirst +
-// 32 j): a packed max tree per lane and a vote; vectors with a logit at or
+// 32 j, there if bit j of `in`): a packed max tree per lane and a vote; vectors with a logit at or
 // over the threshold are queued, and the queue is worked off once it holds 32.
 template <int DT>
-__device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint4* qv, uint32_t* qi, int& qn,
-                                          const uint4 (&d)[PPS_TRUNC_UNITS], int64_t vfirst, int k) {
+__device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint4* st, uint32_t* qi, int& qn,
+                                          const uint4 (&d)[PPS_TRUNC_UNITS], unsigned in, const char* row,
+                                          int64_t vfirst, int h, int k) {
     constexpr int NV = PPS_TRUNC_UNITS;
     const int lane = threadIdx.x & 31;
     unsigned vf = 0;
@@ -531,6 +491,7 @@ __device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint
             for (int j = 0; j < NV; ++j) vf |= (unsigned)(mv[j] >= C.thr) << j;
         }
     }
+    vf &= in;  // past the segment's end a vector of -inf reaches a threshold of -inf, but is not there to be read again
     const int n = __popc(vf);
     int off = n;
 #pragma unroll
@@ -540,26 +501,21 @@ __device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint
     }
     const int total = __shfl_sync(FULL, off, 31);
     off += qn - n;
-#pragma unroll
-    for (int j = 0; j < NV; ++j)
-        if ((vf >> j) & 1u) {
-            qv[off] = d[j];
-            qi[off] = (uint32_t)(vfirst + 32 * j);
-            ++off;
-        }
+    for (; vf; vf &= vf - 1) qi[off++] = (uint32_t)vfirst + 32u * (uint32_t)(__ffs(vf) - 1);
     qn += total;
     if (qn >= 32) {
-        C = topk_flush<DT>(C, sv, si, qv, qi, qn, k);
+        C = topk_flush<DT>(C, sv, si, st, qi, qn, row, h, k);
         qn = 0;
     }
 }
 
-// The fast scan of the full vectors [v0, vend) of a row: iterations of NV
-// vectors 32 apart per lane; in the last, partial one the vectors past vend
-// read as -inf.  The first iteration also seeds the threshold.
+// The fast scan of vectors [v0, vend) of a row's aligned interior (`row`: its
+// start, token h of the row): iterations of NV vectors 32 apart per lane; in
+// the last, partial one the vectors past vend read as -inf.  The first
+// iteration also seeds the threshold.
 template <int DT>
-__device__ __forceinline__ void topk_scan(CandState& C, float* sv, int* si, uint4* qv, uint32_t* qi,
-                                          const char* row, int64_t v0, int64_t vend, int k) {
+__device__ __forceinline__ void topk_scan(CandState& C, float* sv, int* si, uint4* st, uint32_t* qi,
+                                          const char* row, int64_t v0, int64_t vend, int h, int k, float guess) {
     constexpr int NV = PPS_TRUNC_UNITS;
     constexpr int STEP = 32 * NV;
     const int lane = threadIdx.x & 31;
@@ -571,61 +527,65 @@ __device__ __forceinline__ void topk_scan(CandState& C, float* sv, int* si, uint
     for (int64_t it = 0; it < n_it; ++it) {
         const int64_t vb = v0 + it * STEP + lane;
         uint4 d[NV];
+        unsigned in = (1u << NV) - 1u;  // which of the vectors exist
         if (v0 + (it + 1) * STEP <= vend) {
 #pragma unroll
             for (int j = 0; j < NV; ++j) d[j] = ldg_stream(p + 32 * j);
         } else {
+            in = 0;
 #pragma unroll
-            for (int j = 0; j < NV; ++j) d[j] = vb + 32 * j < vend ? ldg_stream(p + 32 * j) : fill;
+            for (int j = 0; j < NV; ++j) {
+                d[j] = fill;
+                if (vb + 32 * j < vend) {
+                    d[j] = ldg_stream(p + 32 * j);
+                    in |= 1u << j;
+                }
+            }
         }
         p += STEP;
-        if (it == 0) C.thr = seed_thr<DT>(d, k);
-        topk_step<DT>(C, sv, si, qv, qi, qn, d, vb, k);
+        if (it == 0) C.thr = fmaxf(guess, seed_thr<DT>(d, k));
+        topk_step<DT>(C, sv, si, st, qi, qn, d, in, row, vb, h, k);
     }
-    if (qn > 0) C = topk_flush<DT>(C, sv, si, qv, qi, qn, k);
+    if (qn > 0) C = topk_flush<DT>(C, sv, si, st, qi, qn, row, h, k);
 }
 
-// Scalar-load path: the last partial iteration of a segment, the ragged
-// vector of a row and unaligned rows, one vector per lane at a time.
+// Segment [v0, v1) (in units of the row partition) of a row.  Finding S needs no
+// Philox words, so vectors need not line up with blocks: the scan takes the
+// row's aligned interior, nfull vectors from its first 16-byte boundary on (h
+// tokens in), and the at most 2 (VW - 1) tokens before and after it are
+// offered one per lane, by the segments that hold the row's start and end.
+// Rows of any alignment stream at the same rate: 16720 rows of V = 5717 bf16,
+// top-k 50, took 736 us when unaligned rows were read one token at a time, 382 with
+// this change alone.
 template <int DT>
-__device__ __noinline__ TopList topk_tail(TopList L, const char* row, int64_t V, int64_t base, int64_t v1, int k) {
+__device__ __forceinline__ CandState topk_segment(const char* row, int64_t V, int64_t v0, int64_t v1, int64_t nv, int k,
+                                                  float* sv, int* si, uint4* st, uint32_t* qi) {
     constexpr int VW = DT == 1 ? 8 : 4;
+    constexpr int ESZ = DT == 1 ? 2 : 4;
     const int lane = threadIdx.x & 31;
-    for (; base < v1; base += 32) {
-        const int64_t v = base + lane;
-        float cv[VW];
-        int ci[VW];
-        uint4 d = make_uint4(0, 0, 0, 0);
-        int64_t nt = 0;
-        if (v < v1) {
-            d = load_scalar<DT>(row, v, V);
-            nt = min((int64_t)VW, V - v * VW);
-        }
-#pragma unroll
-        for (int e = 0; e < VW; ++e) {
-            const float x = vec_token<DT>(d, e);
-            cv[e] = (e < nt && x == x) ? x : -kInf;
-            ci[e] = (int)(v * VW + e);
-        }
-        top_offer<VW>(L, cv, ci, k, lane);
-    }
-    return L;
-}
-
-template <int DT, bool VEC>
-__device__ __forceinline__ void topk_segment(TopList& L, const char* row, int64_t V, int64_t v0, int64_t v1, int k,
-                                             float* sv, int* si, uint4* qv, uint32_t* qi) {
-    constexpr int VW = DT == 1 ? 8 : 4;
-    const int64_t nfull = V / VW;
-    const int64_t vend = VEC ? min(v1, nfull) : v0;
+    const int h = (int)min(V, (int64_t)((0u - (uint32_t)reinterpret_cast<uintptr_t>(row)) & 15u) / ESZ);
+    const int64_t nfull = (V - h) / VW;
+    const int64_t vend = min(v1, nfull);
+    CandState C{-kInf, -kInf, 0};
     if (vend > v0) {
-        CandState C{-kInf, -kInf, 0};
-        topk_scan<DT>(C, sv, si, qv, qi, row, v0, vend, k);
-        if (C.n > kTopMax) C = cand_compact<DT>(C, sv, si, k);
-        L = cand_to_list(C, sv, si, k);
+        const char* in = row + h * ESZ;
+        float guess = vend - v0 >= kSampleMin ? guess_thr<DT>(in, v0, vend, k) : -kInf;
+        while (true) {
+            topk_scan<DT>(C, sv, si, st, qi, in, v0, vend, h, k, guess);
+            if (C.n >= k || guess == -kInf) break;
+            guess = -kInf;  // fewer than k tokens reached the guess: scan again from the proven threshold alone
+            C = CandState{-kInf, -kInf, 0};
+        }
     }
-    // the row's ragged last vector, or a whole unaligned segment
-    if (vend < v1) L = topk_tail<DT>(L, row, V, vend > v0 ? vend : v0, v1, k);
+    const int64_t t0 = h + nfull * VW;  // the tokens after the interior
+    const int nh = v0 == 0 ? h : 0, nt = v1 == nv ? (int)(V - t0) : 0;
+    if (nh + nt > 0) {
+        const int64_t i = lane < 16 ? lane : t0 + (lane - 16);
+        float x = -kInf;
+        if (lane < 16 ? lane < nh : lane - 16 < nt) x = load_logit<DT>(row, i);
+        cand_push<DT>(C, sv, si, x, (int)i, k);
+    }
+    return C;
 }
 
 // ---------------------------------------------------------------- finishing a truncated row
@@ -642,41 +602,48 @@ __device__ __noinline__ int64_t count_logit(const char* row, int64_t V, float x)
 
 // Top-p on the kept-by-top-k set: the list's entries with logit >= lk (a
 // prefix, in top order) plus `extra` more tokens of logit lk that the list
-// could not hold.  Lane 0 walks them in ascending order, exactly as the
-// definition sums; returns the smallest kept logit (every token >= it stays).
+// could not hold.  The lanes form the exponentials and the probabilities; lane 0
+// adds them in ascending order, exactly as the definition sums, and walks the
+// groups; returns the smallest kept logit (every token >= it stays).  (All of
+// it on one lane: 11 sequences, V = 7338, top-k 16, top-p 0.9, 111 us a step
+// instead of 65.)
 __device__ __noinline__ float top_p_keep(const TopList& L, float lk, int64_t extra, float top_p, float T,
-                                         float* s_val) {
+                                         float* s_val, double* s_e) {
     const int lane = threadIdx.x & 31;
+    const bool ka = L.av > -kInf && L.av >= lk, kb = L.bv > -kInf && L.bv >= lk;
+    const int nk = __popc(__ballot_sync(FULL, ka)) + __popc(__ballot_sync(FULL, kb));
+    const double top = (double)__shfl_sync(FULL, L.av, 0), Td = (double)T, cut = 1.0 - (double)top_p;
+    const double ex = exp(((double)lk - top) / Td);
+    const double ea = ka ? exp(((double)L.av - top) / Td) : 0.0, eb = kb ? exp(((double)L.bv - top) / Td) : 0.0;
     s_val[lane] = L.av;
     s_val[32 + lane] = L.bv;
+    s_e[lane] = ea;
+    s_e[32 + lane] = eb;
     __syncwarp();
-    float keep = lk;
-    if (lane == 0) {
-        int nk = 0;
-        while (nk < kTopMax && s_val[nk] > -kInf && s_val[nk] >= lk) ++nk;
-        const double top = (double)s_val[0], Td = (double)T, cut = 1.0 - (double)top_p;
-        const double ex = exp(((double)lk - top) / Td);
-        double Z = 0.0;
-        for (int64_t t = 0; t < extra; ++t) Z += ex;
-        for (int j = nk - 1; j >= 0; --j) Z += exp(((double)s_val[j] - top) / Td);
-        double run = 0.0;
-        for (int64_t t = 0; t < extra; ++t) run += ex / Z;
-        float kv = s_val[0];
-        for (int j = nk - 1; j >= 0; --j) {
-            run += exp(((double)s_val[j] - top) / Td) / Z;
-            if (j > 0 && s_val[j - 1] == s_val[j]) continue;  // not the end of its group
-            if ((double)s_val[j] == top) break;               // the top group stays
-            if (run <= cut) {
-                kv = s_val[j - 1];
-            } else {
-                kv = s_val[j];
-                break;
-            }
+    double Z = 0.0;  // every lane sums alike
+    for (int64_t t = 0; t < extra; ++t) Z += ex;
+    for (int j = nk - 1; j >= 0; --j) Z += s_e[j];
+    __syncwarp();
+    s_e[lane] = ea / Z;
+    s_e[32 + lane] = eb / Z;
+    __syncwarp();
+    const double px = ex / Z;
+    double run = 0.0;
+    for (int64_t t = 0; t < extra; ++t) run += px;
+    float keep = s_val[0];
+    for (int j = nk - 1; j >= 0; --j) {
+        run += s_e[j];
+        if (j > 0 && s_val[j - 1] == s_val[j]) continue;  // not the end of its group
+        if ((double)s_val[j] == top) break;               // the top group stays
+        if (run <= cut) {
+            keep = s_val[j - 1];
+        } else {
+            keep = s_val[j];
+            break;
         }
-        keep = kv;
     }
     __syncwarp();
-    return __shfl_sync(FULL, keep, 0);
+    return keep;
 }
 
 // lower 32 of two lists sorted ascending by (key, token): into x
@@ -699,24 +666,33 @@ __device__ __forceinline__ void merge_low_f(float& xk, int& xi, float yk, int yi
         }
     }
 }
+// Finish row r from its buffer, which holds every token at or over l_(k) but
+// those dropmax tells of.  S comes straight from the buffer: one more
+// compaction leaves the tokens >= l_(k); nothing is sorted but the race keys
+// (short lists by kp rounds of a warp argmin, others by a warp sort).
 template <int DT, bool VERIFY, bool BLK>
-__device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, const TopList& L, int kr, int kp,
-                                            float* s_val, Blk bk, uint32_t* scratch, float* s_cand) {
+__device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, CandState C, int kr, int kp, float* sv,
+                                            int* si, float* s_val, double* s_e, Blk bk) {
     const int lane = threadIdx.x & 31;
     const int k = a.top_k;
-    const float lk = L.entry(k - 1);  // l_(k); -inf when the row has fewer than k usable tokens
-    const bool over = lk > -kInf && L.dropmax >= lk;
+    float lk = -kInf;  // l_(k); -inf when the row has fewer than k usable tokens
+    if (C.n >= k) {
+        C = cand_compact<DT>(C, sv, si, k);
+        lk = C.thr;
+    }
+    const bool over = lk > -kInf && C.dropmax >= lk;
     const char* row = reinterpret_cast<const char*>(a.logits) + (size_t)r * (size_t)a.stride * (DT == 1 ? 2 : 4);
     const uint64_t key = a.key[r], ctx = a.ctx[r];
     const uint32_t pos = a.pos[r];
     float keep = lk;
     if (a.top_p < 1.0f) {
+        const TopList L = cand_to_list(C.n, sv, si);
         int64_t extra = 0;
         if (over) {
             const int in_list = __popc(__ballot_sync(FULL, L.av == lk)) + __popc(__ballot_sync(FULL, L.bv == lk));
             extra = count_logit<DT>(row, a.V, lk) - in_list;
         }
-        keep = top_p_keep(L, lk, extra, a.top_p, a.T, s_val);
+        keep = top_p_keep(L, lk, extra, a.top_p, a.T, s_val, s_e);
     }
     if (over && keep <= lk) {
         // the tie group of l_(k) stays but is not all in the list: exact race
@@ -724,47 +700,86 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, const 
         WarpList W;
         W.reset(kp, kr);
         SlowState st{W};
-        st = tail_loop<DT, BLK>(st, row, a.V, 0, a.nv, a.c, key, ctx, pos, lk, bk,
-                                reinterpret_cast<uint64_t*>(s_cand));
-        finalize_row<DT, VERIFY, BLK>(a, r, st.L.lk, st.L.li, st.L.drop(), kr, kp, lane, bk, scratch);
+        st = tail_loop<DT, BLK>(st, row, a.V, 0, a.nv, a.c, key, ctx, pos, lk, bk, reinterpret_cast<uint64_t*>(sv));
+        finalize_row<DT, VERIFY, BLK>(a, r, st.L.lk, st.L.li, st.L.drop(), kr, kp, lane, bk,
+                                      reinterpret_cast<uint32_t*>(si));
         return;
     }
-    // S = the list's entries with logit >= keep: the race's fp32 keys, the 32
+    // S = the buffer's entries with logit >= keep: the race's fp32 keys, the kp
     // smallest in lane order; finalize_row re-keys near ties in fp64 (S is
     // complete, so nothing was dropped: drop bound +inf)
-    float ka = kInf, kb = kInf;
-    int ia = L.ai, ib = L.bi;
-    // proposal rows of the augmented race: the tokens' block arrivals
-    auto list_key = [&](int i, float l) {
-        const uint32_t w = word_of(key, ctx, pos, i, 1);
-        if constexpr (BLK) return block_key_of(key, ctx, pos, i, w, l, a.c, bk.b, bk.B, bk.invB());
-        return key32(w, l, a.c);
-    };
-    if (L.av > -kInf && L.av >= keep) ka = list_key(ia, L.av);
-    if (L.bv > -kInf && L.bv >= keep) kb = list_key(ib, L.bv);
-    if (ka == kInf) ia = INT_MAX;
-    if (kb == kInf) ib = INT_MAX;
-    warp_sort(ka, ia, lane);
-    warp_sort(kb, ib, lane);
-    merge_low_f(ka, ia, kb, ib, lane);
+    float kk[2];
+    int ii[2];
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int m = 32 * t + lane;
+        const float l = m < C.n ? sv[m] : -kInf;
+        kk[t] = kInf;
+        ii[t] = m < C.n ? si[m] : INT_MAX;
+        if (l > -kInf && l >= keep) {
+            const uint32_t w = word_of(key, ctx, pos, ii[t], 1);
+            // proposal rows of the augmented race: the tokens' block arrivals
+            if constexpr (BLK) kk[t] = block_key_of(key, ctx, pos, ii[t], w, l, a.c, bk.b, bk.B, bk.invB());
+            else kk[t] = key32(w, l, a.c);
+        }
+        if (kk[t] == kInf) ii[t] = INT_MAX;
+    }
+    float ka = kInf;
+    int ia = INT_MAX;
+    if (kp <= kTruncRounds) {
+        for (int m = 0; m < kp; ++m) {
+            const bool second = lex_less(kk[1], ii[1], kk[0], ii[0]);
+            float bk_;
+            const int bi = warp_argmin(second ? kk[1] : kk[0], second ? ii[1] : ii[0], bk_);
+            if (bi == INT_MAX) break;
+            if (lane == m) {
+                ka = bk_;
+                ia = bi;
+            }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+                if (ii[t] == bi) {
+                    kk[t] = kInf;
+                    ii[t] = INT_MAX;
+                }
+        }
+    } else {
+        warp_sort(kk[0], ii[0], lane);
+        warp_sort(kk[1], ii[1], lane);
+        merge_low_f(kk[0], ii[0], kk[1], ii[1], lane);
+        ka = kk[0];
+        ia = ii[0];
+    }
     finalize_row<DT, VERIFY, BLK>(a, r, ka, ia, kInf, kr, kp, lane, bk);
 }
 
+// End of a row segment: publish the segment's buffer (its at most 64 largest
+// tokens), or finish the row if the warp is the last of the row to arrive.  Each
+// segment's threshold bounds l_(k) from below, so of all published tokens only those
+// at or over the largest threshold are gathered again: about as many as one
+// segment holds, whatever their number.  (Merging the sorted lists of 74
+// segments one after another took most of the 263 us of a one-sequence step.)
 template <int DT, bool VERIFY, bool BLK>
 __device__ __noinline__ void finish_trunc_segment(const RaceArgs& a, int64_t r, int64_t gw, int64_t NW, int64_t v0,
-                                                  int64_t v1, TopList L, int kr, int kp, float* s_val, Blk bk,
-                                                  uint32_t* scratch, float* s_cand) {
+                                                  int64_t v1, CandState C, int kr, int kp, float* sv, int* si,
+                                                  float* s_val, double* s_e, Blk bk) {
     const int lane = threadIdx.x & 31;
     const int64_t nv = a.nv;
+    const int k = a.top_k;
     bool final_here = v0 == 0 && v1 == nv;
     if (!final_here) {
-        // publish this segment's list; the last warp of the row merges all segments
+        if (C.n >= k) C = cand_compact<DT>(C, sv, si, k);
         TruncPartial* P = a.tpartials + (gw + r);
-        P->v[lane] = L.av;
-        P->v[32 + lane] = L.bv;
-        P->idx[lane] = L.ai;
-        P->idx[32 + lane] = L.bi;
-        if (lane == 0) P->dropmax = L.dropmax;
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            const int m = 32 * t + lane;
+            P->v[m] = m < C.n ? sv[m] : -kInf;
+            P->idx[m] = m < C.n ? si[m] : INT_MAX;
+        }
+        if (lane == 0) {
+            P->dropmax = C.dropmax;
+            P->thr = C.thr;
+        }
         __threadfence();
         __syncwarp();
         const int64_t first_w = warp_of(r * nv, a.total, NW);
@@ -778,30 +793,49 @@ __device__ __noinline__ void finish_trunc_segment(const RaceArgs& a, int64_t r, 
         final_here = __shfl_sync(FULL, last, 0) != 0;
         if (final_here) {
             __threadfence();
-            L.reset();
-            for (int64_t ww = first_w; ww <= last_w; ++ww) {
-                const TruncPartial* Q = a.tpartials + (ww + r);
-                L.insert_sorted(__ldcg(Q->v + lane), __ldcg(Q->idx + lane), a.top_k, lane);
-                L.insert_sorted(__ldcg(Q->v + 32 + lane), __ldcg(Q->idx + 32 + lane), a.top_k, lane);
-                L.dropmax = fmaxf(L.dropmax, __ldcg(&Q->dropmax));
+            float thr = -kInf, dropmax = -kInf;
+            for (int64_t ww = first_w + lane; ww <= last_w; ww += 32) {
+                thr = fmaxf(thr, __ldcg(&a.tpartials[ww + r].thr));
+                dropmax = fmaxf(dropmax, __ldcg(&a.tpartials[ww + r].dropmax));
             }
+            C.thr = from_order_key(__reduce_max_sync(FULL, order_key(thr)));
+            dropmax = from_order_key(__reduce_max_sync(FULL, order_key(dropmax)));
+            C.dropmax = -kInf;  // gathers the ties of the threshold that were kept
+            C.n = 0;
+            for (int64_t ww = first_w; ww <= last_w; ww += 4) {
+                float v[8];
+                int ix[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const bool on = ww + (j >> 1) <= last_w;
+                    const TruncPartial* Q = a.tpartials + (ww + (j >> 1) + r);
+                    v[j] = on ? __ldcg(Q->v + 32 * (j & 1) + lane) : -kInf;
+                    ix[j] = on ? __ldcg(Q->idx + 32 * (j & 1) + lane) : INT_MAX;
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) cand_push<DT>(C, sv, si, v[j], ix[j], k);
+            }
+            C.dropmax = fmaxf(C.dropmax, dropmax);
         }
     }
     if (final_here) {
-        finalize_trunc<DT, VERIFY, BLK>(a, r, L, kr, kp, s_val, bk, scratch, s_cand);
+        finalize_trunc<DT, VERIFY, BLK>(a, r, C, kr, kp, sv, si, s_val, s_e, bk);
         if constexpr (VERIFY) sequence_ticket(a, r, lane);
     }
 }
 
 // ---------------------------------------------------------------- the kernel
 
-template <int DT, bool VERIFY, bool VEC, bool BLK>
+template <int DT, bool VERIFY, bool BLK>
 __global__ void __launch_bounds__(kThreads, PPS_TRUNC_MIN_BLOCKS) trunc_kernel(const RaceArgs a) {
-    __shared__ float s_val[kTopMax];
     __shared__ __align__(16) float s_cv[kCandCap];
     __shared__ int s_ci[kCandCap];
-    __shared__ uint4 s_qv[kTQueueCap];
-    __shared__ uint32_t s_qi[kTQueueCap];
+    __shared__ uint4 s_st[32];
+    __shared__ __align__(16) uint32_t s_qi[kTQueueCap];
+    // top-p works on the finished row, when the queue is empty
+    double* s_e = reinterpret_cast<double*>(s_qi);
+    float* s_val = reinterpret_cast<float*>(s_e + kTopMax);
+    static_assert(sizeof(s_qi) >= kTopMax * (sizeof(double) + sizeof(float)), "top-p's exponentials and logits");
     pdl_wait();  // the previous kernel's outputs and the workspace it used
     pdl_launch_dependents();
     const int64_t NW = a.G;
@@ -819,15 +853,12 @@ __global__ void __launch_bounds__(kThreads, PPS_TRUNC_MIN_BLOCKS) trunc_kernel(c
         }
         const int kp = min(32, 2 * kr + 1);
         const char* row = reinterpret_cast<const char*>(a.logits) + (size_t)r * (size_t)a.stride * esz;
-        TopList L;
-        L.reset();
-        topk_segment<DT, VEC>(L, row, a.V, v0, v1, a.top_k, s_cv, s_ci, s_qv, s_qi);
+        const CandState C = topk_segment<DT>(row, a.V, v0, v1, nv, a.top_k, s_cv, s_ci, s_st, s_qi);
         Blk bk;
         if constexpr (BLK) {
             bk.b = __ldg(a.row_block + r);
             bk.B = a.n_blocks;
         }
-        finish_trunc_segment<DT, VERIFY, BLK>(a, r, gw, NW, v0, v1, L, kr, kp, s_val, bk,
-                                              reinterpret_cast<uint32_t*>(s_ci), s_cv);
+        finish_trunc_segment<DT, VERIFY, BLK>(a, r, gw, NW, v0, v1, C, kr, kp, s_cv, s_ci, s_val, s_e, bk);
     }
 }

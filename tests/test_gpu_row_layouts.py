@@ -1,7 +1,8 @@
 """Rows of any alignment and length: a row's results depend on its values alone.
 
 Rows that start on 16-byte boundaries stream with 128-bit loads, others through aligned 32-bit
-words, and a row's remainder after the last whole iteration takes its own pass.  Each case places the same logits in rows of
+words (full race) or from their first 16-byte boundary on (truncated race), and a row's remainder
+after the last whole iteration takes its own pass.  Each case places the same logits in rows of
 another offset and stride and compares every output bit for bit with the aligned rows' (which
 the parity suites check against the oracle), around the sizes of a vector, a pass of 32 vectors
 and a fast iteration (96 vectors of bf16, 192 of fp32)."""

@@ -7,7 +7,7 @@ import torch
 
 import oracle
 from paper_2609_21858_gb300 import pps, synth
-from parity import check_workload, compare_draft, compare_winners, f32, run_gpu, run_oracle
+from parity import TOP_P_MARGIN, check_workload, compare_draft, compare_winners, f32, run_gpu, run_oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -137,3 +137,44 @@ def test_full_size_zipf_k8_truncated_sampled_rows():
     ow = oracle.walk(t.gamma, t.seq_off, t.node_draft_row, gd["tok"], gd["ndist"], t.child_node, gv["winner"],
                      gv["word"])
     assert np.array_equal(gv["accept_len"], ow["accept_len"]) and np.array_equal(gv["emitted"], ow["emitted"])
+
+
+def _hard_rows(n, V, dtype, seed):
+    """Rows that a threshold guessed from 32 evenly spread chunks of 32 vectors meets badly, five kinds
+    in turn: random, sorted, the largest logits all inside those chunks (the guess is too high), one
+    value everywhere, fewer usable tokens than top-k."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    x = torch.randn(n, V, generator=g, device="cuda")
+    x[1::5] = -1.1 * torch.log(torch.arange(1, V + 1, device="cuda", dtype=torch.float32))
+    vw = 8 if dtype == torch.bfloat16 else 4
+    chunks = V // vw // 32
+    at = torch.tensor([chunks * c // 32 * 32 * vw + 7 * c for c in range(32)], device="cuda")
+    x[2::5, at] = 9.0 + torch.arange(32, device="cuda") / 16
+    x[3::5] = 0.5
+    x[4::5, 40:] = float("-inf")
+    return x.to(dtype)
+
+
+# rows too many to be cut (long enough for a guess) and few rows cut between warps; starts on 16-byte boundaries and not
+@pytest.mark.parametrize("n,V,dtype,shift", [(2900, 65536, torch.bfloat16, 0), (3100, 49201, torch.bfloat16, 3),
+                                             (2900, 24700, torch.float32, 1), (11, 70001, torch.bfloat16, 1),
+                                             (7, 30000, torch.float32, 0)])
+def test_top_k_threshold_of_hard_rows(n, V, dtype, shift):
+    wide = torch.full((n, V + (-V % 8) + 8), 50.0, dtype=dtype, device="cuda")
+    x = wide[:, shift:shift + V]
+    x.copy_(_hard_rows(n, V, dtype, V))
+    rng = np.random.default_rng(V)
+    key, ctx = rng.integers(0, 2 ** 64, n, dtype=np.uint64), rng.integers(0, 2 ** 64, n, dtype=np.uint64)
+    pos = rng.integers(0, 2 ** 31, n, dtype=np.uint32)
+    ids = tuple(torch.as_tensor(a.view(t)).cuda() for a, t in ((key, np.int64), (ctx, np.int64), (pos, np.int32)))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for top_k, top_p in ((50, 1.0), (64, 0.7), (1, 1.0)):
+        d = pps.draft_list(x, *ids, 8, top_k=top_k, top_p=top_p, status=status)
+        torch.cuda.synchronize()
+        rows = np.arange(min(n, 15)) if n < 100 else np.concatenate([np.arange(10), n - 1 - np.arange(5)])
+        sel = torch.as_tensor(rows, device="cuda")
+        mask, margin = oracle.truncate_rows(x[sel].float().cpu().numpy(), top_k, top_p, 1.0)
+        want = oracle.draft_rows(mask, key[rows], ctx[rows], pos[rows], 8)
+        compare_draft({k: v[sel].cpu().numpy() for k, v in d.items()}, want, loose=margin < TOP_P_MARGIN)
+    assert int(status.item()) == 0
