@@ -11,11 +11,11 @@
 // tensor memory, so no logits row is ever written to HBM.
 //
 // GEMM.  One CTA per SM, warp-specialised: warp 0 issues TMA loads of
-// 128 x 64 hidden tiles and 256 x 64 weight tiles (128-byte swizzle) into a
-// 4-stage shared-memory ring; one thread of warp 1 issues tcgen05.mma
-// (M = 128, N = 256, K = 16, bf16 -> fp32) into one of two 256-column
-// accumulators in tensor memory; warps 2..9 read the finished accumulator
-// with tcgen05.ld (thread = one row, 128 columns each) while the next tile
+// 128 x 64 hidden tiles and 256 x 64 (128 x 64 for a single row block) weight
+// tiles (128-byte swizzle) into a 4 (6) stage shared-memory ring; one thread of
+// warp 1 issues tcgen05.mma (M = 128, N = 256 or 128, K = 16, bf16 -> fp32) into
+// one of two accumulators in tensor memory; warps 2..9 read the finished accumulator
+// with tcgen05.ld (thread = one row, half the columns each) while the next tile
 // accumulates in the other.  CTA c owns row block c % MB and the c / MB-th
 // slice of the vocabulary, so the MB CTAs of a slice read the same weight
 // tiles at the same time (they stay in L2) and a thread's row stays the same
@@ -41,24 +41,30 @@
 namespace lm {
 
 constexpr int BM = 128;                                // rows per tile (TMEM lanes)
-constexpr int BN = 256;                                // vocabulary columns per tile
 constexpr int BK = 64;                                 // reduction step: 64 bf16 = one 128-byte swizzle row
-constexpr int kStages = 4;
 constexpr int kEpiWarps = 8;
 constexpr int kLmThreads = 32 * (2 + kEpiWarps);       // TMA warp, MMA warp, 8 epilogue warps
 constexpr int kStageA = BM * BK * 2;                   // 16 KB
-constexpr int kStageB = BN * BK * 2;                   // 32 KB
-constexpr int kStageBytes = kStageA + kStageB;
-constexpr int kTmemCols = 2 * BN;                      // two fp32 accumulators
 constexpr int kSmCap = 160;                            // slices x row blocks never exceed this (nor the SM count)
 constexpr int kRoomyLists = 32;                        // partial lists per row that the workspace always has room for
 constexpr int kLaneLists = (2 * kSmCap + 31) / 32;     // partial lists per lane of the wide finishing kernel
-constexpr int kLmSmem = kStages * kStageBytes + 1024 /* alignment */ + 256 /* barriers, flags */;
+constexpr int kLmRing = 192 * 1024;                    // the ring of stages
+constexpr int kLmSmem = kLmRing + 1024 /* alignment */ + 256 /* barriers, flags */;
 constexpr uint32_t kLmWaitLimit = 1u << 22;
 
-// instruction descriptor of tcgen05.mma kind::f16: fp32 accumulator (bits 4-5),
-// bf16 A and B (7-9, 10-12), both K-major (15, 16 = 0), N >> 3 (17-22), M >> 4 (24-28)
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+// what depends on the tile width BN (vocabulary columns): 256, or 128 for a single row block (schedule)
+template <int BN>
+struct Tile {
+    static constexpr int kStageB = BN * BK * 2;  // 32 or 16 KB
+    static constexpr int kStageBytes = kStageA + kStageB;
+    static constexpr int kStages = kLmRing / kStageBytes;  // 4 or 6
+    static constexpr int kTmemCols = 2 * BN;               // two fp32 accumulators
+    // instruction descriptor of tcgen05.mma kind::f16: fp32 accumulator (bits 4-5),
+    // bf16 A and B (7-9, 10-12), both K-major (15, 16 = 0), N >> 3 (17-22), M >> 4 (24-28)
+    static constexpr uint32_t kIdesc =
+        (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    static_assert(kStages * kStageBytes <= kLmRing && 8 * (2 * kStages + 4) + 20 <= 256, "ring and barriers fit");
+};
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -122,12 +128,12 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 // D (tmem) = A (smem) x B (smem)^T [+ D]
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t accumulate) {
+__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(kIdesc), "r"(accumulate)
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // thread t of the warp reads lane (taddr lane + t), 32 consecutive 32-bit columns
@@ -179,7 +185,8 @@ struct LmArgs {
     int64_t n_rows, V, d;
     int MB;  // row blocks of BM rows
     int S;   // vocabulary slices per row block
-    int NT;  // vocabulary tiles of BN columns
+    int BN;  // vocabulary columns per tile (Tile)
+    int NT;  // vocabulary tiles
     int KB;  // reduction steps of BK
     // store epilogue: logits [n_rows, ldo] fp32
     float* out;
@@ -349,12 +356,13 @@ struct RaceEpi {
 
 namespace lm {
 
-// Shared memory: kStages x (A tile 16 KB | B tile 32 KB), 1024-byte aligned,
+// Shared memory: kStages x (A tile 16 KB | B tile 32 or 16 KB), 1024-byte aligned,
 // then the mbarriers full[s], empty[s], tfull[2], tempty[2], the abort flag
 // and the tensor-memory address written by tcgen05.alloc.
-template <class Epi>
+template <class Epi, int BN>
 __global__ void __launch_bounds__(kLmThreads, 1)
     lmhead_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const LmArgs a) {
+    constexpr int kStages = Tile<BN>::kStages, kStageBytes = Tile<BN>::kStageBytes, kTmemCols = Tile<BN>::kTmemCols;
     extern __shared__ uint8_t lm_smem_raw[];
     const uint32_t raw = smem_u32(lm_smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
@@ -441,7 +449,8 @@ __global__ void __launch_bounds__(kLmThreads, 1)
                     const uint64_t db = sw128_desc(base + s * kStageBytes + kStageA);
 #pragma unroll
                     for (int k = 0; k < BK / 16; ++k)
-                        tc_mma(d_tmem, da + 2u * (uint32_t)k, db + 2u * (uint32_t)k, (kb | k) != 0 ? 1u : 0u);
+                        tc_mma(d_tmem, da + 2u * (uint32_t)k, db + 2u * (uint32_t)k, Tile<BN>::kIdesc,
+                               (kb | k) != 0 ? 1u : 0u);
                     tc_commit(empty(s));  // frees the stage once these MMAs have read it
                     ++it;
                 }
@@ -450,7 +459,7 @@ __global__ void __launch_bounds__(kLmThreads, 1)
             }
         }
     } else {
-        // ---- epilogue: thread = row m0 + 32 q + lane, columns [128 half, 128 half + 128) of each tile
+        // ---- epilogue: thread = row m0 + 32 q + lane, columns [BN/2 half, BN/2 half + BN/2) of each tile
         const int q = warp & 3, half = (warp - 2) >> 2;
         const int64_t row = (int64_t)m0 + 32 * q + lane;
         Epi epi;
@@ -464,12 +473,12 @@ __global__ void __launch_bounds__(kLmThreads, 1)
             tc_fence_after();
             const int64_t n0 = (int64_t)t * BN;
 #pragma unroll 1
-            for (int ch = 0; ch < 4; ++ch) {
-                const uint32_t col = (uint32_t)(half * 128 + ch * 32);
+            for (int ch = 0; ch < BN / 64; ++ch) {
+                const uint32_t col = (uint32_t)(half * (BN / 2) + ch * 32);
                 uint32_t v[32];
                 tmem_ld32(tmem + acc * BN + ((uint32_t)(32 * q) << 16) + col, v);
                 tmem_wait_ld();
-                if (ch == 3) {
+                if (ch == BN / 64 - 1) {
                     // the accumulator is in registers: hand it back to the MMA warp
                     tc_fence_before();
                     __syncwarp();
@@ -692,23 +701,35 @@ static bool make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+template <class Epi, int BN>
+static cudaError_t launch_gemm_bn(const CUtensorMap& tA, const CUtensorMap& tB, const LmArgs& a, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(lmhead_kernel<Epi, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLmSmem);
+    if (e != cudaSuccess) return e;
+    lmhead_kernel<Epi, BN><<<a.MB * a.S, kLmThreads, kLmSmem, st>>>(tA, tB, a);
+    return cudaGetLastError();
+}
 template <class Epi>
 static cudaError_t launch_gemm(const CUtensorMap& tA, const CUtensorMap& tB, const LmArgs& a, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(lmhead_kernel<Epi>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLmSmem);
-    if (e != cudaSuccess) return e;
-    lmhead_kernel<Epi><<<a.MB * a.S, kLmThreads, kLmSmem, st>>>(tA, tB, a);
-    return cudaGetLastError();
+    return a.BN == 128 ? launch_gemm_bn<Epi, 128>(tA, tB, a, st) : launch_gemm_bn<Epi, 256>(tA, tB, a, st);
 }
 
 // The schedule: MB row blocks x S vocabulary slices, S = SMs / MB (at least 1, at most NT), so that
 // every SM has a CTA.  With few row blocks the pass is bound by reading the weights once from HBM,
 // which takes the whole chip: the two launches of one sequence (41 rows of d = 4096, 33 of d = 2048,
-// V = 128256: 1.58 GB) take 317 us = 5.0 TB/s on 152 slices, 1131 us on 16.
+// V = 128256: 1.58 GB) take 303 us = 5.2 TB/s, 1131 us on 16 slices.  A single row block takes
+// 128-column tiles where they shorten the longest slice (501 tiles of 256 on 152 slices: four, or seven
+// halves; 319 -> 303 us for one sequence, 328 -> 320 us for the 123 rows of three); where they do not
+// (V = 66624, 117 rows: 239 against 254 us) and with more row blocks, where the tensor cores count, 256.
+// (One equal run of tiles per SM across row blocks, walked in phase, was slower than whole slices: 2642
+// against 2516 us for 64 sequences, although it uses 152 SMs instead of 136 and 147.)
 static void schedule(LmArgs& a) {
     a.MB = (int)((a.n_rows + BM - 1) / BM);
-    a.NT = (int)((a.V + BN - 1) / BN);
     a.KB = (int)((a.d + BK - 1) / BK);
-    a.S = min(max(1, min(device_sm_count(), kSmCap) / max(1, a.MB)), a.NT);
+    const int S = max(1, min(device_sm_count(), kSmCap) / max(1, a.MB));
+    auto run = [&](int bn) { return ((a.V + bn - 1) / bn + S - 1) / S; };  // tiles of the longest run
+    a.BN = a.MB == 1 && run(128) < 2 * run(256) ? 128 : 256;
+    a.NT = (int)((a.V + a.BN - 1) / a.BN);
+    a.S = min(S, a.NT);
 }
 
 }  // namespace lm
@@ -732,7 +753,7 @@ cudaError_t launch_lmhead_logits(const void* hidden, int64_t ldh, const void* we
     a.ldo = ldo;
     lm::schedule(a);
     CUtensorMap tA, tB;
-    if (!lm::make_map(&tA, hidden, n_rows, d, ldh, lm::BM) || !lm::make_map(&tB, weight, V, d, ldw, lm::BN))
+    if (!lm::make_map(&tA, hidden, n_rows, d, ldh, lm::BM) || !lm::make_map(&tB, weight, V, d, ldw, a.BN))
         return cudaErrorInvalidValue;
     return lm::launch_gemm<lm::StoreEpi>(tA, tB, a, st);
 }
@@ -754,7 +775,7 @@ cudaError_t launch_lmhead_race(const void* hidden, int64_t ldh, const void* weig
     a.partials = static_cast<lm::LmPartial*>(ws);
     lm::schedule(a);
     CUtensorMap tA, tB;
-    if (!lm::make_map(&tA, hidden, a.n_rows, d, ldh, lm::BM) || !lm::make_map(&tB, weight, a.V, d, ldw, lm::BN))
+    if (!lm::make_map(&tA, hidden, a.n_rows, d, ldh, lm::BM) || !lm::make_map(&tB, weight, a.V, d, ldw, a.BN))
         return cudaErrorInvalidValue;
     cudaError_t e = a.K <= 1 ? lm::launch_gemm<lm::RaceEpi<3>>(tA, tB, a, st)
                              : lm::launch_gemm<lm::RaceEpi<lm::kLmKP>>(tA, tB, a, st);

@@ -190,11 +190,12 @@ def test_fused_race_matches_the_oracle_on_dyadic_operands():
         np.testing.assert_allclose(v["score_sum"].cpu().numpy(), ow["score_sum"], rtol=1e-5)
 
 
-# row blocks of 128 rows x vocabulary slices of 256-column tiles over the SMs: one row on every
+# row blocks of 128 rows x vocabulary slices of 256 or 128-column tiles over the SMs: one row on every
 # slice, a whole and a just begun second block, fewer tiles than SMs (one tile a slice, the last one
-# ragged), and both sides of 32 partial lists per row (10 and 11 blocks)
+# ragged), both sides of 32 partial lists per row (9 and 10 blocks: 16 and 15 slices on 152 SMs), and a
+# single block of a vocabulary large enough for 256-column tiles (the others of one block take 128)
 @pytest.mark.parametrize("n,V", [(1, 39000), (41, 38913), (128, 700), (129, 20000), (520, 9001), (1030, 6000),
-                                 (1153, 6000), (1281, 5000)])
+                                 (1153, 6000), (1281, 5000), (100, 320001)])
 def test_fused_race_over_many_slices_equals_the_unfused_path(n, V):
     h, w = _normal(n, V, 72, n + V)
     _, (key, ctx, pos) = _ids(n, n)
