@@ -15,7 +15,7 @@
 // conservative fp32 filter that rejects almost every token with one ex2 and
 // a few multiply-pipe operations (pps_device.cuh).  Survivors get the fp32 key
 // and enter a per-warp sorted list of kp = min(32, 2k+1) entries (one per
-// lane).  Lists of a row are merged with warp bitonic merges.  The finished
+// lane).  Lists of a row are merged with warp argmin rounds.  The finished
 // list proves its own completeness (every dropped token has a key above the
 // k-th key plus both error bounds) and re-orders near-ties with the fp64 key
 // s = ln E - l/T, so the selected tokens and their order are those of the
@@ -60,7 +60,9 @@
 #define PPS_VF_MAXK 4  // draft rows with lists up to this long stream like verify rows (one test per vector)
 #endif
 #ifndef PPS_SEG_CAP
-#define PPS_SEG_CAP 30  // at most this many warp segments per row (small launches; keeps <= 32 partial lists)
+// at most this many warp segments per row (launches of few rows; keeps <= kMaxLists partial lists): one
+// sequence of the benchmark tree takes 46.5 us a step, 50 with 30 segments
+#define PPS_SEG_CAP 60
 #endif
 
 namespace pps {
@@ -98,12 +100,19 @@ __device__ __forceinline__ float unord_key(uint32_t u) {
 }
 // smallest of the warp's values (none NaN)
 __device__ __forceinline__ float warp_min(float f) { return unord_key(__reduce_min_sync(FULL, ord_key(f))); }
-// the k-th smallest of the warp's 32 values (none NaN): the smallest by one
-// redux.min, others bit by bit
+// the k-th smallest of the warp's 32 values (none NaN): a few by redux.min
+// rounds that drop one value each, others bit by bit
 __device__ __forceinline__ float warp_kth(float f, int k) {
-    if (k == 1) return warp_min(f);
-    const uint32_t u = ord_key(f);
+    uint32_t u = ord_key(f);
     uint32_t res = 0;
+    if (k <= 12) {
+#pragma unroll 1
+        while (true) {
+            res = __reduce_min_sync(FULL, u);
+            if (--k == 0) return unord_key(res);
+            if ((int)(threadIdx.x & 31) == __ffs(__ballot_sync(FULL, u == res)) - 1) u = 0xffffffffu;
+        }
+    }
 #pragma unroll 1
     for (int b = 31; b >= 0; --b) {
         const uint32_t cand = res | (1u << b);
@@ -147,38 +156,6 @@ __device__ __forceinline__ void warp_sort(float& k, int& i, int lane) {
             }
         }
     }
-}
-
-// merge a sorted list (lk, li) with a sorted batch (ok, oi); keep the kp smallest.
-// Returns (warp-uniform) the smallest key it discards: the (kp+1)-th of the union.
-__device__ __forceinline__ float warp_merge(float& lk, int& li, float ok, int oi, int kp, int lane) {
-    float rk = __shfl_sync(FULL, ok, 31 - lane);
-    int ri = __shfl_sync(FULL, oi, 31 - lane);
-    float dropk = rk;
-    if (lex_less(rk, ri, lk, li)) {
-        dropk = lk;
-        lk = rk;
-        li = ri;
-    }
-    // (lk, li) is now bitonic and holds the 32 smallest of the union
-#pragma unroll 1
-    for (int stride = 16; stride > 0; stride >>= 1) {
-        float xk = __shfl_xor_sync(FULL, lk, stride);
-        int xi = __shfl_xor_sync(FULL, li, stride);
-        bool lower = (lane & stride) == 0;
-        bool o_less = lex_less(xk, xi, lk, li);
-        if (lower ? o_less : (!o_less && !(xk == lk && xi == li))) {
-            lk = xk;
-            li = xi;
-        }
-    }
-    if (kp < 32) dropk = fminf(dropk, __shfl_sync(FULL, lk, kp & 31));
-    dropk = warp_min(dropk);
-    if (lane >= kp) {
-        lk = kInf;
-        li = INT_MAX;
-    }
-    return dropk;
 }
 
 __device__ __forceinline__ void warp_sort_d(double& k, int& i, int lane) {
@@ -1395,101 +1372,71 @@ __device__ __noinline__ void sequence_ticket(const RaceArgs& a, int64_t r, int l
     __syncwarp();
 }
 
-// Merge the partial lists of warps first_w..last_w of row r into (lk, li) and
-// lower theta_drop to a bound on every key the merged list leaves out.  The
-// partials were written by warps all over the GPU (L2 round trips of a
-// microsecond or so), so they are loaded kMergeBatch at a time, all loads of a
-// batch in flight together, and a batch is merged as a tree (independent pairs
-// first), so that a small launch with many warps per row does not pay one
-// round trip and one dependent merge per partial.  Merging two sorted lists
-// keeps the kp smallest of their union and reports the smallest key it drops,
-// so every key left out of the result is >= the minimum of both lists' drop
-// bounds and the dropped keys.
-constexpr int kMergeBatch = 8;
-
-__device__ __forceinline__ void merge_partials(const RaceArgs& a, int64_t r, int64_t first_w, int64_t last_w, int kp,
-                                               int lane, float& lk, int& li, float& theta_drop) {
-    for (int64_t w0 = first_w; w0 <= last_w; w0 += kMergeBatch) {
-        const int nb = (int)min((int64_t)kMergeBatch, last_w - w0 + 1);  // warp-uniform
-        float pk[kMergeBatch], pd[kMergeBatch];
-        int pi[kMergeBatch];
-#pragma unroll
-        for (int b = 0; b < kMergeBatch; ++b) {
-            pk[b] = kInf;
-            pi[b] = INT_MAX;
-            pd[b] = kInf;
-            if (b < nb) {
-                const Partial* Q = a.partials + (w0 + b + r);
-                pk[b] = __ldcg(Q->key + lane);
-                pi[b] = __ldcg(Q->idx + lane);
-                pd[b] = __ldcg(&Q->theta_drop);
-            }
-        }
-        // tree: (0,1) (2,3) (4,5) (6,7), then (0,2) (4,6), then (0,4); empty lists are skipped
-#pragma unroll
-        for (int s = 1; s < kMergeBatch; s <<= 1) {
-#pragma unroll
-            for (int b = 0; b + s < kMergeBatch; b += 2 * s) {
-                if (b + s < nb) {
-                    const float dk = warp_merge(pk[b], pi[b], pk[b + s], pi[b + s], kp, lane);
-                    pd[b] = fminf(fminf(pd[b], pd[b + s]), dk);
-                }
-            }
-        }
-        const float dk = warp_merge(lk, li, pk[0], pi[0], kp, lane);
-        theta_drop = fminf(theta_drop, fminf(pd[0], dk));
-    }
-}
-
-// Merge by selection rounds, for at most 32 partial lists: list j is staged in
-// row j of s_k / s_i (entry e at [j * 32 + e], e < kp) by asynchronous 16-byte
-// copies that every lane issues for its whole list before one wait (one L2
-// round trip for the lot), lane j holds the head of list j, and each of kp
-// rounds moves the warp's smallest head (key, token) to entry m of the merged
-// list and advances its lane.  One warp argmin per output entry replaces one
-// dependent bitonic merge per list.  Tokens are unique across the lists
+// Merge row r's P <= kMaxLists partial lists by selection rounds: the first
+// entries of the lists (all kp of them for up to 32 lists, 16 beyond) are staged
+// in s_k / s_i by asynchronous 16-byte copies that every lane issues for its
+// lists before one wait (one L2 round trip for the lot); lane j holds the heads
+// of lists j and j + 32, and each of kp rounds moves the warp's smallest head (key, token)
+// to entry m of the merged list and advances its list (past the staged entries,
+// which hardly happens, from L2).  One warp argmin per output entry replaces one
+// dependent merge per list.  Tokens are unique across the lists
 // (disjoint segments of one row), so only the owner's head matches the
 // winner.  The smallest head left over is the smallest listed key dropped.
-// s_k and s_i are 16-byte aligned.
+// s_k and s_i are 16-byte aligned, 1024 entries each.
 __device__ __forceinline__ void copy16_async(void* smem, const void* gmem) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
                  "l"(gmem)
                  : "memory");
 }
 
+constexpr int kMaxLists = 64;
+static_assert(PPS_SEG_CAP + 2 <= kMaxLists, "a row meets at most this many warps");
+
 __device__ __noinline__ void merge_rounds(const RaceArgs& a, int64_t r, int64_t first_w, int P, int kp, int lane,
                                           float* s_k, int* s_i, float& lk, int& li, float& theta_drop) {
+    const int stride = P <= 32 ? 32 : 16, staged = min(kp, stride);
+    const Partial* Q = a.partials + (first_w + lane + r);
     float th = kInf;
-    if (lane < P) {
-        const Partial* Q = a.partials + (first_w + lane + r);
-        th = __ldcg(&Q->theta_drop);
-        for (int e = 0; e < kp; e += 4) {
-            copy16_async(s_k + lane * 32 + e, Q->key + e);
-            copy16_async(s_i + lane * 32 + e, Q->idx + e);
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+        if (lane + 32 * j < P) {
+            th = fminf(th, __ldcg(&Q[32 * j].theta_drop));
+            const int at = (lane + 32 * j) * stride;
+            for (int e = 0; e < staged; e += 4) {
+                copy16_async(s_k + at + e, Q[32 * j].key + e);
+                copy16_async(s_i + at + e, Q[32 * j].idx + e);
+            }
         }
-    }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
-    int h = 0;
-    float hk = lane < P ? s_k[lane * 32] : kInf;
-    int hi = lane < P ? s_i[lane * 32] : INT_MAX;
+    int h[2] = {0, 0}, hi[2];
+    float hk[2];
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const bool on = lane + 32 * j < P;
+        hk[j] = on ? s_k[(lane + 32 * j) * stride] : kInf;
+        hi[j] = on ? s_i[(lane + 32 * j) * stride] : INT_MAX;
+    }
     lk = kInf;
     li = INT_MAX;
     for (int m = 0; m < kp; ++m) {
+        const bool second = lex_less(hk[1], hi[1], hk[0], hi[0]);
         float bk;
-        const int bi = warp_argmin(hk, hi, bk);
+        const int bi = warp_argmin(second ? hk[1] : hk[0], second ? hi[1] : hi[0], bk);
         if (bi == INT_MAX) break;  // fewer listed entries than kp (warp-uniform)
         if (lane == m) {
             lk = bk;
             li = bi;
         }
-        if (hi == bi) {
-            ++h;
-            hk = h < kp ? s_k[lane * 32 + h] : kInf;
-            hi = h < kp ? s_i[lane * 32 + h] : INT_MAX;
-        }
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+            if (hi[j] == bi) {
+                const int n = ++h[j], at = (lane + 32 * j) * stride + n;
+                hk[j] = n < staged ? s_k[at] : n < kp ? __ldcg(Q[32 * j].key + n) : kInf;
+                hi[j] = n < staged ? s_i[at] : n < kp ? __ldcg(Q[32 * j].idx + n) : INT_MAX;
+            }
     }
-    theta_drop = fminf(theta_drop, warp_min(fminf(hk, th)));
+    theta_drop = fminf(theta_drop, warp_min(fminf(fminf(hk[0], hk[1]), th)));
     __syncwarp();
 }
 
@@ -1530,10 +1477,7 @@ __device__ __noinline__ void finish_segment(const RaceArgs& a, int64_t r, int64_
             lk = kInf;
             li = INT_MAX;
             theta_drop = kInf;
-            if (last_w - first_w < 32)
-                merge_rounds(a, r, first_w, (int)(last_w - first_w + 1), kp, lane, s_mk, s_mi, lk, li, theta_drop);
-            else
-                merge_partials(a, r, first_w, last_w, kp, lane, lk, li, theta_drop);
+            merge_rounds(a, r, first_w, (int)(last_w - first_w + 1), kp, lane, s_mk, s_mi, lk, li, theta_drop);
         }
     }
     if (final_here) {
@@ -1640,7 +1584,7 @@ int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk, int64_t
     // (64 sequences of 3 rows of V = 1000, fp32: 45 -> 33 us a step)
     const int64_t by_size = max((total + kMinVecsPerWarp - 1) / kMinVecsPerWarp, n_rows);
     if (by_size < g) g = by_size;
-    if (PPS_SEG_CAP > 0 && n_rows > 0 && n_rows * PPS_SEG_CAP < g) g = n_rows * PPS_SEG_CAP;
+    if (n_rows > 0 && n_rows * PPS_SEG_CAP < g) g = n_rows * PPS_SEG_CAP;
     if (n_rows > 0) {
         // every warp gets at least one unit (one fast iteration of a row), so every
         // warp a row's counter waits for streams part of it

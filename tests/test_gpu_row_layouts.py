@@ -10,7 +10,9 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from paper_2609_21858_gb300 import pps
+from parity import compare_draft
 
 pytestmark = pytest.mark.gpu
 
@@ -89,3 +91,25 @@ def test_results_do_not_depend_on_the_rows_place(dtype, offset, pad):
             a = pps.draft_hetero(y, *ids, blk, 4, status=status, **kw)
             assert torch.equal(a, pps.draft_hetero(z, *ids, blk, 4, status=status, **kw)), V
         assert int(status.item()) == 0, V
+
+
+# a row cut between as many warps as it can be (60), and between a few; the whole list (K = 32: more
+# entries than the merge stages of each list) in one warp's segment, or spread
+@pytest.mark.parametrize("n,V,dtype", [(1, 128256, BF), (2, 40000, BF), (3, 70001, F32)])
+@pytest.mark.parametrize("where", ["one", "all"])
+def test_lists_of_rows_cut_between_many_warps(n, V, dtype, where):
+    rng = np.random.default_rng(V + n)
+    x = rng.normal(0, 1, (n, V)).astype(np.float32)
+    if where == "one":
+        x[:, V // 3:V // 3 + 90] += 25.0
+    x = torch.as_tensor(x).to(dtype).cuda()
+    ids = [rng.integers(0, 2 ** 64, n, dtype=np.uint64), rng.integers(0, 2 ** 64, n, dtype=np.uint64),
+           rng.integers(0, 2 ** 31, n, dtype=np.uint32)]
+    dev = [torch.as_tensor(a.view(t)).cuda() for a, t in zip(ids, (np.int64, np.int64, np.int32))]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for K, mode in ((32, pps.DISTINCT), (8, pps.IID), (1, pps.DISTINCT)):
+        d = pps.draft_list(x, *dev, K, mode=mode, status=status)
+        torch.cuda.synchronize()
+        want = oracle.draft_rows(x.float().cpu().numpy(), *ids, K, mode=mode)
+        compare_draft({k: v.cpu().numpy() for k, v in d.items()}, want)
+    assert int(status.item()) == 0
