@@ -15,7 +15,7 @@
  *   runtime.  Outputs are undefined unless the call returned PPS_OK.
  * - Logits rows are `row_stride` elements apart (row_stride >= vocab),
  *   row-major, fp32 or bf16.  Rows whose start is 16-byte aligned are
- *   streamed with 128-bit loads; other layouts take a slower scalar path.
+ *   streamed with 128-bit loads, others with aligned 32-bit ones.
  * - Row identities (pps_row_ids) label the keyed Poisson source G(k, c) of the
  *   paper (Sec. 3.3, Alg. 3 and 4, detector algorithm of App. E): a 64-bit
  *   watermark key, a 64-bit context label Lambda(c) and a 32-bit position.

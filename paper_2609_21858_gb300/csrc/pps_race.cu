@@ -1492,7 +1492,7 @@ __device__ __noinline__ void finish_segment(const RaceArgs& a, int64_t r, int64_
 // race_unit(DT) vectors (the last may be shorter), and warp gw of NW streams the
 // units [gw*U/NW, (gw+1)*U/NW) of the U = n_rows * nb units in row order.  For
 // bf16 rows a unit is one fast-loop iteration, so that a segment ends on an
-// iteration boundary and only a row's ragged end takes the scalar tail
+// iteration boundary and only a row's end takes tail_scan
 // (measured on the bench tree: verify 0.282 -> 0.272 ms, draft 0.248 ->
 // 0.235 ms); fp32 rows keep units of one vector (iteration units made the
 // fp32 tree slower, 7.35 -> 7.73 ms).  A row cut between warps is merged and finished by
@@ -1582,7 +1582,10 @@ int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk, int64_t
     int64_t g = (int64_t)device_sm_count() * o;
     // a warp per row at least: rows of fewer vectors one after another in a warp add up their latencies
     // (64 sequences of 3 rows of V = 1000, fp32: 45 -> 33 us a step)
-    const int64_t by_size = max((total + kMinVecsPerWarp - 1) / kMinVecsPerWarp, n_rows);
+    // (rows of 1024 vectors and more may be cut twice as fine: 12 sequences, V = 18368, 41 -> 38 us; shorter
+    // rows gain nothing from a second warp: V = 1000, fp32, 33 -> 44 us)
+    const int64_t least = n_rows > 0 && total >= 1024 * n_rows ? kMinVecsPerWarp / 2 : kMinVecsPerWarp;
+    const int64_t by_size = max((total + least - 1) / least, n_rows);
     if (by_size < g) g = by_size;
     if (n_rows > 0 && n_rows * PPS_SEG_CAP < g) g = n_rows * PPS_SEG_CAP;
     if (n_rows > 0) {
