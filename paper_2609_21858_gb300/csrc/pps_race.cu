@@ -1540,11 +1540,14 @@ __global__ void __launch_bounds__(kThreads, BLK ? PPS_BLOCK_MIN_BLOCKS : PPS_RAC
         // A one-token draft list is a target race, and a list of a few tokens is close to one:
         // such rows stream like verify rows (one filter test per vector; measured: lists of up
         // to 4 gain, lists of 8 lose).  A row cut between warps shares its filter bound (verify,
-        // short-list draft and proposal rows: on longer lists the shared bound saves too little).
+        // short-list bf16 draft and proposal rows: on longer lists the shared bound saves too little,
+        // and in fp32 draft rows, half the tokens to a byte, the loop without its read is faster:
+        // 41216 rows of V = 152064 4.93 -> 4.63 ms, 16 sequences of that tree 854 -> 834 us a step;
+        // the benchmark's bf16 tree takes 488 us with it, 497 without).
         const bool one = VERIFY || (!BLK && kr <= PPS_VF_MAXK);
         uint32_t* slot = nullptr;
         if constexpr (PPS_ROWBOUND)
-            if ((one || BLK) && a.row_bound && (v0 > 0 || v1 < nv)) slot = a.row_bound + r;
+            if ((VERIFY || BLK || DT == 1) && (one || BLK) && a.row_bound && (v0 > 0 || v1 < nv)) slot = a.row_bound + r;
         // fp32 rows always stream with the vector test: one loop in the kernel, not two alike
         // (two cost the fp32 draft launch 12%: 340 -> 381 us)
         constexpr bool kVec = VERIFY || DT == 0;
