@@ -21,6 +21,11 @@ import torch
 from . import pps
 
 
+def _as_stored(x, mine, n: int) -> bool:
+    """Whether x is n values of mine's dtype on its device, so that a copy into it changes nothing but the place."""
+    return isinstance(x, torch.Tensor) and x.dtype is mine.dtype and x.device == mine.device and x.shape == (n,)
+
+
 class TreeBuilder:
     """Buffers for the dynamic IID trees of n_seq sequences (reused by every `run`)."""
 
@@ -68,11 +73,15 @@ class TreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_list (IID) and one pps_tree_expand."""
         K = self.K
-        for mine, root, x in zip(self._ids[0], self._root, (root_key, root_ctx, root_pos)):
-            mine.copy_(x)
-            root.copy_(x)
-        self._ids[0][3].fill_(K)
         nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
+        for mine, root, node, x in zip(self._ids[0], self._root, nodes.values(), (root_key, root_ctx, root_pos)):
+            if _as_stored(x, mine, self.n_seq):
+                mine.copy_(x)
+                root.copy_(x)
+            else:  # a scalar or one root for all; the write by index refuses any other dtype, device or length
+                mine[:] = x
+                node[self.roots] = x
+        self._ids[0][3].fill_(K)
         for d in range(self.gamma):
             key, ctx, pos, k = self._ids[d]
             out = self._out[d]
@@ -153,12 +162,16 @@ class HeteroTreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_hetero and one pps_hetero_expand."""
         B = self.B
-        for mine, root, x in zip(self._ids[0], self._root, (root_key, root_ctx, root_pos)):
-            mine.view(self.n_seq, B).copy_(x[:, None].expand(-1, B))
-            root.copy_(x)
-        self._ids[0][3].zero_()
         lists = dict(tok=self.list_tok, ndist=self.list_nd, child=self.child_node)
         nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
+        for mine, root, node, x in zip(self._ids[0], self._root, nodes.values(), (root_key, root_ctx, root_pos)):
+            if _as_stored(x, mine, self.n_seq):
+                mine.view(self.n_seq, B).copy_(x[:, None].expand(-1, B))
+                root.copy_(x)
+            else:  # the write by index refuses another dtype, device or length
+                mine[:] = x.repeat_interleave(B)
+                node[self.roots] = x
+        self._ids[0][3].zero_()
         for d in range(self.gamma):
             key, ctx, pos, owner = self._ids[d]
             blk, tok = self._blk_tok[d]

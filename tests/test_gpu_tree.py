@@ -84,3 +84,13 @@ def test_dynamic_tree_matches_the_oracle(K, gamma, V, dtype):
     assert np.array_equal(v["emitted"].cpu().numpy(), ow["emitted"])
     # the root keeps K paths: every sequence emitted at least its root's winner
     assert np.all(v["n_emitted"].cpu().numpy() >= 1)
+
+
+@pytest.mark.parametrize("builder", [tree.TreeBuilder, tree.HeteroTreeBuilder])
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_roots_in_host_memory_are_refused(builder, which):
+    ids = [torch.arange(3).cuda(), torch.arange(3).cuda(), torch.arange(3, dtype=torch.int32).cuda()]
+    ids[which] = ids[which].cpu()
+    with pytest.raises(RuntimeError):
+        builder(3, 2, 2).run(*ids, lambda d, *_: torch.zeros(6 if builder is tree.HeteroTreeBuilder or d else 3, 50,
+                                                             device="cuda"))
