@@ -92,9 +92,11 @@ int pps_philox_rounds(void);
  * n_seq sequences (n_seq = 0 for pps_draft_list).  The workspace holds
  * per-row partial candidate lists, arrival counters and the shared filter
  * bounds of rows cut between CTAs; it must be zeroed once
- * before its first use (pps_workspace_clear or cudaMemset) and is left zeroed
- * by every call that returns PPS_OK and runs to completion.  One workspace
- * must not be used by two calls that run concurrently. */
+ * before its first use (pps_workspace_clear or cudaMemset).  A call that
+ * returns PPS_OK and runs to completion leaves its counters and bounds zero
+ * (they lie at the end of the ws_bytes bytes, the lists at the start), so one
+ * workspace, given with the same ws_bytes, serves further calls of the same or
+ * fewer rows.  It must not be used by two calls that run concurrently. */
 size_t pps_workspace_size(int64_t n_rows, int64_t vocab, int32_t K, int32_t n_seq);
 pps_status pps_workspace_clear(void* ws, size_t ws_bytes, pps_stream_t stream);
 

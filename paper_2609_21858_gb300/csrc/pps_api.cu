@@ -1,6 +1,7 @@
 // pps_api.cu -- extern "C" entry points of libpps: argument validation,
 // workspace layout and launches.  Every entry point returns before launching
 // anything when an argument is invalid.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdint>
@@ -15,19 +16,25 @@ namespace pps {
 
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t workspace_bytes(int64_t n_rows, int32_t n_seq) {
-    return align256(kSlotBytes * (size_t)(n_rows + (int64_t)kGridMax)) + align256(sizeof(uint32_t) * 2 * (size_t)n_rows) +
-           align256(sizeof(uint32_t) * (size_t)(n_seq > 0 ? n_seq : 0));
+// A workspace serves calls of any size up to the one it was made for, and only its counters are
+// zero between calls, so no call's partial lists may reach another's counters: the lists start at
+// the buffer's start and the counters end at its end.  Both parts grow with n_rows alone (a call has
+// at most as many sequences as rows), so the lists of n rows end below the counters of any call
+// that fits.
+static size_t list_bytes(int64_t n_rows) { return align256(kSlotBytes * (size_t)(n_rows + (int64_t)kGridMax)); }
+static size_t counter_bytes(int64_t n_rows, int32_t n_seq) {
+    return align256(sizeof(uint32_t) * (2 * (size_t)n_rows + (size_t)std::max(n_rows, (int64_t)n_seq)));
 }
 
-void workspace_carve(void* ws, int64_t n_rows, int32_t n_seq, Partial** partials, uint32_t** row_cnt,
+size_t workspace_bytes(int64_t n_rows, int32_t n_seq) { return list_bytes(n_rows) + counter_bytes(n_rows, n_seq); }
+
+void workspace_carve(void* ws, size_t ws_bytes, int64_t n_rows, int32_t n_seq, Partial** partials, uint32_t** row_cnt,
                      uint32_t** seq_cnt) {
     char* p = static_cast<char*>(ws);
     *partials = reinterpret_cast<Partial*>(p);
-    p += align256(kSlotBytes * (size_t)(n_rows + (int64_t)kGridMax));
+    p += (ws_bytes & ~(size_t)255) - counter_bytes(n_rows, n_seq);
     *row_cnt = reinterpret_cast<uint32_t*>(p);  // [n_rows] arrival counters, then [n_rows] shared row bounds
-    p += align256(sizeof(uint32_t) * 2 * (size_t)n_rows);
-    *seq_cnt = reinterpret_cast<uint32_t*>(p);
+    *seq_cnt = *row_cnt + 2 * n_rows;
 }
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -189,7 +196,7 @@ static pps_status draft_list(const void* q_logits, pps_dtype dtype, int64_t n_ro
     a.out_nd = out_ndistinct;
     a.out_samples = out_samples;
     a.status = status;
-    workspace_carve(ws, n_rows, 0, &a.partials, &a.row_cnt, &a.seq_cnt);
+    workspace_carve(ws, ws_bytes, n_rows, 0, &a.partials, &a.row_cnt, &a.seq_cnt);
     a.row_bound = a.row_cnt + n_rows;
     a.tpartials = reinterpret_cast<TruncPartial*>(a.partials);
     a.top_k = top_k;
@@ -262,7 +269,7 @@ static pps_status verify_tree(const void* p_logits, pps_dtype dtype, int64_t n_n
     a.out_sc = out_score;
     a.out_ss = out_score_sum;
     a.status = status;
-    workspace_carve(ws, n_nodes, n_seq, &a.partials, &a.row_cnt, &a.seq_cnt);
+    workspace_carve(ws, ws_bytes, n_nodes, n_seq, &a.partials, &a.row_cnt, &a.seq_cnt);
     a.row_bound = a.row_cnt + n_nodes;
     a.tpartials = reinterpret_cast<TruncPartial*>(a.partials);
     a.top_k = top_k;
@@ -535,7 +542,7 @@ static pps_status draft_hetero(const void* q_logits, pps_dtype dtype, int64_t n_
         a.row_block = row_block;
         a.n_blocks = n_blocks;
     }
-    workspace_carve(ws, n_rows, 0, &a.partials, &a.row_cnt, &a.seq_cnt);
+    workspace_carve(ws, ws_bytes, n_rows, 0, &a.partials, &a.row_cnt, &a.seq_cnt);
     a.row_bound = a.row_cnt + n_rows;
     a.tpartials = reinterpret_cast<TruncPartial*>(a.partials);
     a.top_k = top_k;

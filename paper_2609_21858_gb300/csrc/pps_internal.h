@@ -116,7 +116,7 @@ inline cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, si
 }
 
 size_t workspace_bytes(int64_t n_rows, int32_t n_seq);
-void workspace_carve(void* ws, int64_t n_rows, int32_t n_seq, Partial** partials, uint32_t** row_cnt,
+void workspace_carve(void* ws, size_t ws_bytes, int64_t n_rows, int32_t n_seq, Partial** partials, uint32_t** row_cnt,
                      uint32_t** seq_cnt);
 
 // launchers (pps_race.cu)

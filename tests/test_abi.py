@@ -302,3 +302,30 @@ def test_lmhead_entry_points_validate_arguments():
         assert verify(**kw) == pps.ERR_INVALID_ARG, kw
     assert verify(wsb=0) == pps.ERR_WORKSPACE
     assert _header_defines()["PPS_LMHEAD_MAX_K"] == pps.LMHEAD_MAX_K
+
+
+def _carve(L, ws_bytes, n_rows, n_seq):
+    """(partial lists, row counters, sequence counters) as offsets in a workspace of ws_bytes bytes."""
+    carve = getattr(L, "_ZN3pps15workspace_carveEPvmliPPNS_7PartialEPPjS5_")
+    carve.argtypes = [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int64, ctypes.c_int32] + [ctypes.c_void_p] * 3
+    carve.restype = None
+    at = [ctypes.c_void_p() for _ in range(3)]
+    base = 1 << 20  # never dereferenced
+    carve(base, ws_bytes, n_rows, n_seq, *(ctypes.addressof(x) for x in at))
+    return [x.value - base for x in at]
+
+
+@pytest.mark.parametrize("n_max", [1, 63, 1000, 16720, 41984])
+@pytest.mark.parametrize("spare", [0, 1, 300])
+def test_no_call_writes_lists_where_a_smaller_call_has_its_counters(n_max, spare):
+    # one slot per row and per warp (at most 16384) of the larger of the two kinds of partial list
+    L = pps.lib()
+    slot, warps = 64 * 8 + 16, 16384
+    wsb = pps.workspace_size(n_max, 0, 1, n_max) + spare
+    for n in sorted({1, n_max // 3 + 1, n_max - 1 or 1, n_max}):
+        for s in (0, 1, n):
+            assert pps.workspace_size(n, 0, 1, s) <= wsb
+            lists, rows, seqs = _carve(L, wsb, n, s)
+            assert lists == 0 and rows % 16 == 0
+            assert rows >= slot * (n_max + warps)
+            assert seqs == rows + 8 * n and seqs + 4 * s <= wsb
