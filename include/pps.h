@@ -417,9 +417,10 @@ pps_status pps_wm_detect(const int32_t* tokens, pps_row_ids ids, int64_t n, int3
  * are limited to K <= PPS_LMHEAD_MAX_K.  A row whose kept candidates cannot
  * prove its list complete (more than one near tie at the k-th key) raises
  * PPS_FLAG_GUARD; PPS_FLAG_TIMEOUT reports a pipeline that gave up waiting
- * (outputs undefined).  The workspace holds the partial lists and the
- * sequence tickets: pps_lmhead_workspace_size bytes, zeroed once before first
- * use (pps_workspace_clear); the calls leave it ready for the next call.
+ * (outputs undefined).  The workspace holds the partial lists and, at its
+ * end, the sequence tickets: pps_lmhead_workspace_size bytes, zeroed once
+ * before first use (pps_workspace_clear); given with the same ws_bytes it
+ * serves further LM-head calls of the same or fewer rows.
  */
 #define PPS_LMHEAD_MAX_K 8
 size_t pps_lmhead_workspace_size(int64_t n_rows, int32_t n_seq);

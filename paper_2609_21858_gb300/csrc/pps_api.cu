@@ -455,8 +455,7 @@ pps_status pps_lmhead_verify_tree(const void* hidden, int64_t ld_hidden, const v
     a.out_sc = out_score;
     a.out_ss = out_score_sum;
     a.status = status;
-    // the sequence tickets follow the partial lists
-    a.seq_cnt = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + lmhead_workspace_bytes(n_nodes, 0));
+    a.seq_cnt = lmhead_tickets(ws, ws_bytes, n_nodes, n_seq);
     return launch_lmhead_race(hidden, ld_hidden, weight, ld_weight, d, a, true, ws, (cudaStream_t)stream) ==
                    cudaSuccess
                ? PPS_OK

@@ -139,6 +139,7 @@ int trunc_grid(int64_t total, int64_t n_rows, int dtype, bool verify, bool blk =
 // the LM-head GEMM with the race in its epilogue (pps_lmhead.cuh, in pps_race.cu).
 // hidden [n_rows, d] and weight [V, d] are bf16 with row strides ldh, ldw elements.
 size_t lmhead_workspace_bytes(int64_t n_rows, int32_t n_seq);
+uint32_t* lmhead_tickets(void* ws, size_t ws_bytes, int64_t n_rows, int32_t n_seq);  // [n_seq], zero between calls
 cudaError_t launch_lmhead_logits(const void* hidden, int64_t ldh, const void* weight, int64_t ldw, int64_t n_rows,
                                  int64_t V, int64_t d, float* out, int64_t ldo, cudaStream_t st);
 cudaError_t launch_lmhead_race(const void* hidden, int64_t ldh, const void* weight, int64_t ldw, int64_t d,

@@ -45,7 +45,7 @@ constexpr int BK = 64;                                 // reduction step: 64 bf1
 constexpr int kEpiWarps = 8;
 constexpr int kLmThreads = 32 * (2 + kEpiWarps);       // TMA warp, MMA warp, 8 epilogue warps
 constexpr int kStageA = BM * BK * 2;                   // 16 KB
-constexpr int kSmCap = 160;                            // slices x row blocks never exceed this (nor the SM count)
+constexpr int kSmCap = 160;                            // slices x row blocks, for up to as many blocks (beyond: one slice)
 constexpr int kRoomyLists = 32;                        // partial lists per row that the workspace always has room for
 constexpr int kLaneLists = (2 * kSmCap + 31) / 32;     // partial lists per lane of the wide finishing kernel
 constexpr int kLmRing = 192 * 1024;                    // the ring of stages
@@ -734,12 +734,21 @@ static void schedule(LmArgs& a) {
 
 }  // namespace lm
 
-// n_rows x 2 S partial lists: at most 2 BM kSmCap of them, or 2 per row beyond kSmCap row blocks.
-// The size never falls as n_rows grows, so a workspace serves every smaller call too.
+// n_rows x 2 S partial lists from the buffer's start on: at most 2 BM kSmCap of them, or 2 per row
+// beyond kSmCap row blocks.  The sequence tickets end where the buffer ends.  Both parts grow with
+// n_rows alone (a call has at most as many sequences as rows), so the lists of n rows end below the
+// tickets of any call that fits, and a workspace serves every smaller call too.
+static size_t lmhead_ticket_bytes(int64_t n_rows, int32_t n_seq) {
+    const int64_t least = 2 * lm::BM * lm::kSmCap / lm::kRoomyLists;  // fewer rows have the same lists, and the same size
+    return (sizeof(uint32_t) * (size_t)max(least, max(n_rows, (int64_t)n_seq)) + 255) & ~(size_t)255;
+}
 size_t lmhead_workspace_bytes(int64_t n_rows, int32_t n_seq) {
-    auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t lists = (size_t)max((int64_t)2 * lm::BM * lm::kSmCap, n_rows * lm::kRoomyLists);
-    return al(sizeof(lm::LmPartial) * lists) + al(sizeof(uint32_t) * (size_t)(n_seq > 0 ? n_seq : 0));
+    static_assert(sizeof(lm::LmPartial) * lm::kRoomyLists % 256 == 0, "the lists are whole 256-byte units");
+    return sizeof(lm::LmPartial) * lists + lmhead_ticket_bytes(n_rows, n_seq);
+}
+uint32_t* lmhead_tickets(void* ws, size_t ws_bytes, int64_t n_rows, int32_t n_seq) {
+    return reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + (ws_bytes & ~(size_t)255) - lmhead_ticket_bytes(n_rows, n_seq));
 }
 
 cudaError_t launch_lmhead_logits(const void* hidden, int64_t ldh, const void* weight, int64_t ldw, int64_t n_rows,

@@ -329,3 +329,20 @@ def test_no_call_writes_lists_where_a_smaller_call_has_its_counters(n_max, spare
             assert lists == 0 and rows % 16 == 0
             assert rows >= slot * (n_max + warps)
             assert seqs == rows + 8 * n and seqs + 4 * s <= wsb
+
+
+@pytest.mark.parametrize("n_max", [1, 1280, 1281, 20481, 41984])
+def test_no_lmhead_call_writes_lists_where_a_smaller_call_has_its_tickets(n_max):
+    # 128-byte lists: 2 x (160 // row blocks) of them a row, 2 beyond 160 blocks of 128 rows
+    L = pps.lib()
+    tickets = getattr(L, "_ZN3pps14lmhead_ticketsEPvmli")
+    tickets.argtypes = [ctypes.c_void_p, ctypes.c_size_t, ctypes.c_int64, ctypes.c_int32]
+    tickets.restype = ctypes.c_void_p
+    base, wsb = 1 << 20, L.pps_lmhead_workspace_size(n_max, n_max)  # base is never dereferenced
+    lists = max(128 * n * 2 * max(1, 160 // (-(-n // 128))) for n in {1, 128, 1280, 20480, n_max} if n <= n_max)
+    for n in {1, n_max // 3 + 1, n_max}:
+        for s in (1, n):
+            assert L.pps_lmhead_workspace_size(n, s) <= wsb
+            at = tickets(base, wsb, n, s) - base
+            assert at >= lists and at + 4 * s <= wsb
+    assert L.pps_lmhead_workspace_size(1, 0) == L.pps_lmhead_workspace_size(1280, 1280)

@@ -68,3 +68,24 @@ def test_small_calls_after_a_large_one(n, V, dtype, top_k):
             _same(v, _verify(lambda *a, **k: pps.verify_tree(y[:m // 5 * 5], *a, **k), m, jds, None, **kw))
     _same(pps.draft_list(x, *ids, 8, top_k=top_k, ws=ws, status=status), big)
     assert int(status.item()) == 0
+
+
+@pytest.mark.parametrize("n", [129, 1300, 41984])
+def test_small_lmhead_calls_after_a_large_one(n):
+    # 41984 rows: 328 row blocks, two partial lists a row
+    V, d = 700, 64
+    g = torch.Generator(device="cuda")
+    g.manual_seed(n)
+    h = torch.randn(n, d, generator=g, device="cuda").to(BF)
+    w = torch.randn(V, d, generator=g, device="cuda").to(BF)
+    ids = _rows(n, 1, F32, n)[1]
+    ws = pps.lmhead_workspace(n, n)
+    big = pps.lmhead_draft_list(h, w, *ids, 8)
+    _same(pps.lmhead_draft_list(h, w, *ids, 8, ws=ws), big)
+    for m in (1000, 65, 5):
+        m = min(m, n // 5 * 5)
+        jds = [x[:m] for x in ids]
+        _same(pps.lmhead_draft_list(h[:m], w, *jds, 4, ws=ws), pps.lmhead_draft_list(h[:m], w, *jds, 4))
+        call = lambda *a, **k: pps.lmhead_verify_tree(h[:m], w, *a, **k)
+        _same(_verify(call, m, jds, ws), _verify(call, m, jds, None))
+    _same(pps.lmhead_draft_list(h, w, *ids, 8, ws=ws), big)
