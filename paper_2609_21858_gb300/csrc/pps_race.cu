@@ -1048,13 +1048,13 @@ __device__ __noinline__ bool iid_fast(const RaceArgs& a, int64_t r, float lk, in
 // lanes 0..: (dk, li).  Every token whose exact key is at most the row's
 // exact k-th key has a list key within that cut.  Returns false when more
 // tokens than the buffer holds crowd the cut.  `scratch` holds
-// 1 + 2 kRescanCap words.
+// 1 + 2 kRescanCap words.  Tokens with a logit below `floor` take no part
+// (truncated rows: the smallest logit kept).
 constexpr int kRescanCap = 96;
 
 template <int DT, bool BLK>
-__device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau, int kr, int lane, Blk bk,
+__device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau, int lane, Blk bk, float floor,
                                         uint32_t* scratch, double& dk, int& li, int& nvalid) {
-    constexpr int VW = DT == 1 ? 8 : 4;
     const uint64_t key = a.key[r], ctx = a.ctx[r];
     const uint32_t pos = a.pos[r];
     const char* row = reinterpret_cast<const char*>(a.logits) + (size_t)r * (size_t)a.stride * (DT == 1 ? 2 : 4);
@@ -1083,7 +1083,7 @@ __device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau,
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int64_t i = (int64_t)4 * cb + e;
-                    if (i < a.V && v * VW + 4 * h + e < a.V && filter_pass(wq[e], l[e], c, tz)) {
+                    if (i < a.V && !(l[e] < floor) && filter_pass(wq[e], l[e], c, tz)) {
                         float k;
                         if constexpr (BLK)
                             k = block_key_of(key, ctx, pos, i, wq[e], l[e], c, bk.b, bk.B, bk.invB());
@@ -1166,15 +1166,16 @@ __device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau,
         }
     }
     nvalid = take;
-    (void)kr;
     return true;
 }
 
 // Warp 0 finishes row r from its complete list (lk, li) and the drop bound.
-// BLK: the near-tie keys are those of the row's block arrivals.
+// BLK: the near-tie keys are those of the row's block arrivals.  floor: the
+// smallest logit that takes part in the row's race.
 template <int DT, bool VERIFY, bool BLK, class LP>
 __device__ __forceinline__ void finalize_row_lp(const RaceArgs& a, int64_t r, float lk, int li, float theta_drop,
-                                                int kr, int kp, int lane, const LP& lp, Blk bk, uint32_t* scratch) {
+                                                int kr, int kp, int lane, const LP& lp, Blk bk, uint32_t* scratch,
+                                                float floor = -kInf) {
     const int nvalid = __popc(__ballot_sync(FULL, lane < kp && lk < kInf));
     const float tau = nvalid >= kr ? __shfl_sync(FULL, lk, kr - 1) : kInf;
     // list-key error bound (block rows: widened by kBlkErr)
@@ -1190,7 +1191,7 @@ __device__ __forceinline__ void finalize_row_lp(const RaceArgs& a, int64_t r, fl
         // the boundary is crowded: finish the row exactly with one more pass
         double dkr;
         int lir, nvr;
-        if (rescan_row<DT, BLK>(a, r, tau, kr, lane, bk, scratch, dkr, lir, nvr)) {
+        if (rescan_row<DT, BLK>(a, r, tau, lane, bk, floor, scratch, dkr, lir, nvr)) {
             if (lane == 0 && a.status && tau > -kInf && fabsf(tau) > 65536.0f) atomicOr(a.status, PPS_FLAG_LOGIT_RANGE);
             emit_row<DT, VERIFY>(a, r, dkr, (float)dkr, lir, nvr, kr, lane, a.key[r], a.ctx[r], a.pos[r], lp);
             return;
@@ -1234,8 +1235,9 @@ __device__ __forceinline__ void finalize_row_lp(const RaceArgs& a, int64_t r, fl
 // Warp 0 finishes row r of a streamed logits matrix from its complete list.
 template <int DT, bool VERIFY, bool BLK = false>
 __device__ __noinline__ void finalize_row(const RaceArgs& a, int64_t r, float lk, int li, float theta_drop, int kr,
-                                          int kp, int lane, Blk bk = Blk{}, uint32_t* scratch = nullptr) {
-    finalize_row_lp<DT, VERIFY, BLK>(a, r, lk, li, theta_drop, kr, kp, lane, dense_logits<DT>(a, r), bk, scratch);
+                                          int kp, int lane, Blk bk = Blk{}, uint32_t* scratch = nullptr,
+                                          float floor = -kInf) {
+    finalize_row_lp<DT, VERIFY, BLK>(a, r, lk, li, theta_drop, kr, kp, lane, dense_logits<DT>(a, r), bk, scratch, floor);
 }
 
 // vectors per unit of the streaming kernel's row partition (see race_kernel)

@@ -702,7 +702,7 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, CandSt
         SlowState st{W};
         st = tail_loop<DT, BLK>(st, row, a.V, 0, a.nv, a.c, key, ctx, pos, lk, bk, reinterpret_cast<uint64_t*>(sv));
         finalize_row<DT, VERIFY, BLK>(a, r, st.L.lk, st.L.li, st.L.drop(), kr, kp, lane, bk,
-                                      reinterpret_cast<uint32_t*>(si));
+                                      reinterpret_cast<uint32_t*>(si), lk);
         return;
     }
     // S = the buffer's entries with logit >= keep: the race's fp32 keys, the kp

@@ -178,3 +178,51 @@ def test_top_k_threshold_of_hard_rows(n, V, dtype, shift):
         want = oracle.draft_rows(mask, key[rows], ctx[rows], pos[rows], 8)
         compare_draft({k: v[sel].cpu().numpy() for k, v in d.items()}, want, loose=margin < TOP_P_MARGIN)
     assert int(status.item()) == 0
+
+
+def _random_ids(n, seed):
+    rng = np.random.default_rng(seed)
+    ids = (rng.integers(0, 2 ** 64, n, dtype=np.uint64), rng.integers(0, 2 ** 64, n, dtype=np.uint64),
+           rng.integers(0, 2 ** 31, n, dtype=np.uint32))
+    return ids, tuple(torch.as_tensor(a.view(t)).cuda() for a, t in zip(ids, (np.int64, np.int64, np.int32)))
+
+
+def _exactly_the_oracles(x, ids, dev, K, mode, top_k, top_p):
+    """Lists (and, for K = 1, winners) of the truncated rows, near ties included."""
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    d = pps.draft_list(torch.as_tensor(x).cuda(), *dev, K, mode=mode, top_k=top_k, top_p=top_p, status=status)
+    masked, _ = oracle.truncate_rows(x, top_k, f32(top_p), 1.0)
+    want = oracle.draft_rows(masked, *ids, K, mode=mode)
+    assert np.array_equal(d["tok"].cpu().numpy(), want["tok"])
+    assert np.array_equal(d["samples"].cpu().numpy(), want["labels"])
+    if K == 1:
+        n = len(x)
+        off = torch.arange(n + 1, dtype=torch.int32, device="cuda")
+        none = torch.full((n,), -1, dtype=torch.int32, device="cuda")
+        one = torch.zeros(1, 1, dtype=torch.int32, device="cuda")
+        v = pps.verify_tree(torch.as_tensor(x).cuda(), *dev, 1, off, none, one, one[0], one, top_k=top_k, top_p=top_p,
+                            status=status)
+        assert np.array_equal(v["winner"].cpu().numpy(), want["tok"][:, 0])
+    assert int(status.item()) == 0
+
+
+# rows whose tie group at l_(k) overflows the list, the K-th key crowded (so that the row is scanned once
+# more), and 400 tokens just below l_(k), many of them with smaller keys
+@pytest.mark.parametrize("V,top_p", [(2000, 1.0), (2000, 0.9999), (40000, 1.0)])
+@pytest.mark.parametrize("K", [8, 32])
+def test_a_second_scan_of_a_crowded_row_keeps_to_the_truncated_set(K, V, top_p):
+    n, top_k, tied, extra = 16, 40, 150, 20
+    ids, dev = _random_ids(n, 50 + K)
+    rng = np.random.default_rng(V + K)
+    x = np.full((n, V), -20.0, np.float32)
+    for r in range(n):
+        w = oracle.words(*(a[r:r + 1] for a in ids), V)[0]
+        log_e = np.log(-np.log((w + 0.5) * 2.0 ** -32))
+        at = rng.permutation(V)
+        x[r, at[:tied]] = 4.0
+        x[r, at[tied:tied + 400]] = rng.uniform(3.2, 3.9, 400)
+        last = np.sort(log_e[at[:tied]] - 4.0)[K - 1]
+        rest = at[tied + 400:]
+        rest = rest[log_e[rest] - last > 4.001][:extra]  # their logits come to lie above the tie group's
+        x[r, rest] = log_e[rest] - last - rng.uniform(-3e-7, 3e-7, extra)
+    _exactly_the_oracles(x, ids, dev, K, pps.DISTINCT, top_k, top_p)
