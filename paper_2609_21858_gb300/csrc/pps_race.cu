@@ -1039,6 +1039,62 @@ __device__ __noinline__ bool iid_fast(const RaceArgs& a, int64_t r, float lk, in
     return true;
 }
 
+// fp64 race key of token i of logit l (proposal rows: of its block arrival)
+template <bool BLK>
+__device__ __forceinline__ double exact_key(uint64_t key, uint64_t ctx, uint32_t pos, int i, float l, float T, const Blk& bk) {
+    const uint32_t w = word_of(key, ctx, pos, i, 1);
+    if constexpr (BLK) {
+        uint32_t wf;
+        const int J = block_words(key, ctx, pos, i, bk.b, bk.B, wf);
+        return block_key64(w, J, wf, bk.b, bk.B, l, T);
+    } else {
+        return key64(w, l, T);
+    }
+}
+
+// The `take` <= 32 smallest of the warp's 32 x N entries (d, id) in order: lane m receives the m-th.
+template <int N>
+__device__ __forceinline__ void select_exact(double (&d)[N], int (&id)[N], int take, int lane, double& dk, int& li) {
+    dk = (double)INFINITY;
+    li = INT_MAX;
+    for (int m = 0; m < take; ++m) {
+        double bd = d[0];
+        int bi = id[0], bt = 0;
+#pragma unroll
+        for (int t = 1; t < N; ++t)
+            if (lex_less_d(d[t], id[t], bd, bi)) {
+                bd = d[t];
+                bi = id[t];
+                bt = t;
+            }
+        double wd = bd;
+        int wi = bi, wl = lane;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const double od = __shfl_xor_sync(FULL, wd, off);
+            const int oi = __shfl_xor_sync(FULL, wi, off);
+            const int ol = __shfl_xor_sync(FULL, wl, off);
+            if (lex_less_d(od, oi, wd, wi)) {
+                wd = od;
+                wi = oi;
+                wl = ol;
+            }
+        }
+        if (lane == m) {
+            dk = wd;
+            li = wi;
+        }
+        if (lane == wl) {
+#pragma unroll
+            for (int t = 0; t < N; ++t)
+                if (t == bt) {
+                    d[t] = (double)INFINITY;
+                    id[t] = INT_MAX;
+                }
+        }
+    }
+}
+
 // Exact finish of a row whose list could not prove itself complete: tokens
 // crowd its k-th key tau within the error bounds and the 32-entry list has no
 // room left to hold them (always the case for k = 32 on a full list).  One
@@ -1114,58 +1170,11 @@ __device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau,
         id[t] = INT_MAX;
         if (m < n) {
             id[t] = ci[m];
-            const uint32_t w = word_of(key, ctx, pos, id[t], 1);
-            const float l = logit_at<DT>(a, r, id[t]);
-            if constexpr (BLK) {
-                uint32_t wf;
-                const int J = block_words(key, ctx, pos, id[t], bk.b, bk.B, wf);
-                d[t] = block_key64(w, J, wf, bk.b, bk.B, l, a.T);
-            } else {
-                d[t] = key64(w, l, a.T);
-            }
+            d[t] = exact_key<BLK>(key, ctx, pos, id[t], logit_at<DT>(a, r, id[t]), a.T, bk);
         }
     }
-    // the min(n, 32) smallest in order: lane m receives the m-th
-    dk = (double)INFINITY;
-    li = INT_MAX;
-    const int take = min(n, 32);
-    for (int m = 0; m < take; ++m) {
-        double bd = d[0];
-        int bi = id[0], bt = 0;
-#pragma unroll
-        for (int t = 1; t < 3; ++t)
-            if (lex_less_d(d[t], id[t], bd, bi)) {
-                bd = d[t];
-                bi = id[t];
-                bt = t;
-            }
-        double wd = bd;
-        int wi = bi, wl = lane;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double od = __shfl_xor_sync(FULL, wd, off);
-            const int oi = __shfl_xor_sync(FULL, wi, off);
-            const int ol = __shfl_xor_sync(FULL, wl, off);
-            if (lex_less_d(od, oi, wd, wi)) {
-                wd = od;
-                wi = oi;
-                wl = ol;
-            }
-        }
-        if (lane == m) {
-            dk = wd;
-            li = wi;
-        }
-        if (lane == wl) {
-#pragma unroll
-            for (int t = 0; t < 3; ++t)
-                if (t == bt) {
-                    d[t] = (double)INFINITY;
-                    id[t] = INT_MAX;
-                }
-        }
-    }
-    nvalid = take;
+    nvalid = min(n, 32);
+    select_exact<3>(d, id, nvalid, lane, dk, li);
     return true;
 }
 
@@ -1217,15 +1226,7 @@ __device__ __forceinline__ void finalize_row_lp(const RaceArgs& a, int64_t r, fl
     double dk = (double)INFINITY;
     float sk = key_to_s(lk);
     if (need_exact) {
-        if (lane < nvalid) {
-            uint32_t w = word_of(key, ctx, pos, li, 1);
-            if constexpr (BLK) {
-                uint32_t wf;
-                const int J = block_words(key, ctx, pos, li, bk.b, bk.B, wf);
-                dk = block_key64(w, J, wf, bk.b, bk.B, lp(li), a.T);
-            } else
-                dk = key64(w, lp(li), a.T);
-        }
+        if (lane < nvalid) dk = exact_key<BLK>(key, ctx, pos, li, lp(li), a.T, bk);
         warp_sort_d(dk, li, lane);
         sk = (float)dk;
     }

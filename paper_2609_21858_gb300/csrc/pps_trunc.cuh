@@ -25,10 +25,10 @@
 // the tie group stays in S, by the exact fp32 race of pps_race.cu over the
 // tokens with logit >= l_(k).  Otherwise the finishing warp keys the <= 64
 // surviving tokens with the race's fp32 key, keeps the smallest and hands
-// them to finalize_row with a drop bound of +inf (S is complete, nothing was
-// dropped); finalize_row re-keys in fp64 (s = ln E - l/T) every pair closer
+// them to finalize_row, which re-keys in fp64 (s = ln E - l/T) every pair closer
 // than the fp32 error bounds, so the row is emitted exactly like the
-// untruncated race.
+// untruncated race; a row whose K-th key is that close to a key left out takes
+// the fp64 keys of all of S (finish_crowded).
 //
 // A step of the benchmark's tree (top-k 50: 1.21 GB of logits) takes 266 us =
 // 4.6 TB/s, 290 when every row's threshold climbed from the first iteration's and S
@@ -646,11 +646,13 @@ __device__ __noinline__ float top_p_keep(const TopList& L, float lk, int64_t ext
     return keep;
 }
 
-// lower 32 of two lists sorted ascending by (key, token): into x
-__device__ __forceinline__ void merge_low_f(float& xk, int& xi, float yk, int yi, int lane) {
+// lower 32 of two lists sorted ascending by (key, token): into x; returns the lane's key of the upper 32
+__device__ __forceinline__ float merge_low_f(float& xk, int& xi, float yk, int yi, int lane) {
     const float rk = __shfl_sync(FULL, yk, 31 - lane);
     const int ri = __shfl_sync(FULL, yi, 31 - lane);
+    float up = rk;
     if (lex_less(rk, ri, xk, xi)) {
+        up = xk;
         xk = rk;
         xi = ri;
     }
@@ -665,7 +667,33 @@ __device__ __forceinline__ void merge_low_f(float& xk, int& xi, float yk, int yi
             xi = oi;
         }
     }
+    return up;
 }
+
+// Finish a row when more keys crowd its K-th, tau, than the kept list holds: the
+// K smallest of S (the n buffered tokens with logit >= keep) by their fp64 keys.
+template <int DT, bool VERIFY, bool BLK>
+__device__ __noinline__ void finish_crowded(const RaceArgs& a, int64_t r, float tau, int n, float keep, int kr,
+                                            const float* sv, const int* si, Blk bk) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t key = a.key[r], ctx = a.ctx[r];
+    const uint32_t pos = a.pos[r];
+    if (lane == 0 && a.status && fabsf(tau) > 65536.0f) atomicOr(a.status, PPS_FLAG_LOGIT_RANGE);
+    double d[2], dk;
+    int id[2], li, size = 0;
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        const int m = 32 * t + lane;
+        const float l = m < n ? sv[m] : -kInf;
+        const bool in = l > -kInf && l >= keep;
+        id[t] = in ? si[m] : INT_MAX;
+        d[t] = in ? exact_key<BLK>(key, ctx, pos, id[t], l, a.T, bk) : (double)INFINITY;
+        size += __popc(__ballot_sync(FULL, in));
+    }
+    select_exact<2>(d, id, min(size, 32), lane, dk, li);
+    emit_row<DT, VERIFY>(a, r, dk, (float)dk, li, min(size, 32), kr, lane, key, ctx, pos, dense_logits<DT>(a, r));
+}
+
 // Finish row r from its buffer, which holds every token at or over l_(k) but
 // those dropmax tells of.  S comes straight from the buffer: one more
 // compaction leaves the tokens >= l_(k); nothing is sorted but the race keys
@@ -706,8 +734,8 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, CandSt
         return;
     }
     // S = the buffer's entries with logit >= keep: the race's fp32 keys, the kp
-    // smallest in lane order; finalize_row re-keys near ties in fp64 (S is
-    // complete, so nothing was dropped: drop bound +inf)
+    // smallest in lane order, and `left`, the smallest key of the others.  When it
+    // is beyond the K-th key's error bounds, finalize_row re-keys near ties in fp64
     float kk[2];
     int ii[2];
 #pragma unroll
@@ -724,7 +752,7 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, CandSt
         }
         if (kk[t] == kInf) ii[t] = INT_MAX;
     }
-    float ka = kInf;
+    float ka = kInf, left;
     int ia = INT_MAX;
     if (kp <= kTruncRounds) {
         for (int m = 0; m < kp; ++m) {
@@ -743,12 +771,20 @@ __device__ __noinline__ void finalize_trunc(const RaceArgs& a, int64_t r, CandSt
                     ii[t] = INT_MAX;
                 }
         }
+        left = fminf(kk[0], kk[1]);
     } else {
         warp_sort(kk[0], ii[0], lane);
         warp_sort(kk[1], ii[1], lane);
-        merge_low_f(kk[0], ii[0], kk[1], ii[1], lane);
+        left = merge_low_f(kk[0], ii[0], kk[1], ii[1], lane);
         ka = kk[0];
         ia = ii[0];
+        if (lane >= kp) left = fminf(left, ka);
+    }
+    left = warp_min(left);
+    const float tau = __shfl_sync(FULL, ka, kr - 1), eb = BLK ? kBlkErr : 0.f;
+    if (left < kInf && tau > -kInf && !(left > tau + key_err_bound(tau) + key_err_bound(left) + 2.0f * eb)) {
+        finish_crowded<DT, VERIFY, BLK>(a, r, tau, C.n, keep, kr, sv, si, bk);
+        return;
     }
     finalize_row<DT, VERIFY, BLK>(a, r, ka, ia, kInf, kr, kp, lane, bk);
 }

@@ -226,3 +226,49 @@ def test_a_second_scan_of_a_crowded_row_keeps_to_the_truncated_set(K, V, top_p):
         rest = rest[log_e[rest] - last > 4.001][:extra]  # their logits come to lie above the tie group's
         x[r, rest] = log_e[rest] - last - rng.uniform(-3e-7, 3e-7, extra)
     _exactly_the_oracles(x, ids, dev, K, pps.DISTINCT, top_k, top_p)
+
+
+def _crowded(ids, V, usable, lo, hi, K, seed):
+    """fp32 rows whose `usable` tokens (the rest at -30) have their keys of ranks lo .. hi - 1 within 1e-6
+    of the K-th smallest one, in an order that only 64 bits tell."""
+    rng = np.random.default_rng(seed)
+    key, ctx, pos = ids
+    x = np.full((len(key), V), -30.0, np.float32)
+    for r in range(len(key)):
+        at = rng.choice(V, usable, replace=False)
+        log_e = np.log(-np.log((oracle.words(key[r:r + 1], ctx[r:r + 1], pos[r:r + 1], V)[0, at] + 0.5) * 2.0 ** -32))
+        l = rng.normal(5, 1.5, usable)
+        order = np.argsort(log_e - l)
+        s = (log_e - l)[order]
+        l[order[lo:hi]] = log_e[order[lo:hi]] - s[K - 1] - rng.uniform(-3e-7, 3e-7, hi - lo)
+        x[r, at] = l
+    return x
+
+
+# more keys within the fp32 error bounds of the K-th than the kept list (2 K + 1 entries, at most 32) holds
+@pytest.mark.parametrize("V", [3000, 40000])
+@pytest.mark.parametrize("K,mode", [(1, pps.DISTINCT), (8, pps.DISTINCT), (8, pps.IID), (15, pps.DISTINCT),
+                                    (31, pps.DISTINCT), (32, pps.DISTINCT), (32, pps.IID)])
+def test_lists_of_rows_crowded_at_the_last_key(K, mode, V):
+    ids, dev = _random_ids(24, K)
+    x = _crowded(ids, V, 64, max(0, K - 3), min(64, 2 * K + 10), K, K + V)
+    _exactly_the_oracles(x, ids, dev, K, mode, 64, 1.0)
+
+
+def test_proposals_of_rows_crowded_at_the_first_key():
+    n, V, B, usable = 24, 900, 3, 40
+    ids, dev = _random_ids(n, 9)
+    block = (np.arange(n) % B).astype(np.int32)
+    rng = np.random.default_rng(10)
+    x = np.full((n, V), -30.0, np.float32)
+    for r in range(n):
+        at = rng.choice(V, usable, replace=False)
+        log_e = np.log([oracle.block_e(*(int(a[r]) for a in ids), int(i), int(block[r]), B) for i in at])
+        l = rng.normal(5, 1.5, usable)
+        first = np.argsort(log_e - l)[:10]
+        l[first] = log_e[first] - (log_e - l).min() - rng.uniform(-3e-7, 3e-7, 10)
+        x[r, at] = l
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    got = pps.draft_hetero(torch.as_tensor(x).cuda(), *dev, torch.as_tensor(block).cuda(), B, top_k=usable, status=status)
+    assert np.array_equal(got.cpu().numpy(), oracle.block_draft_rows(x, *ids, block, B)[0])
+    assert int(status.item()) == 0
