@@ -453,17 +453,21 @@ __device__ __noinline__ CandState topk_flush(CandState C, float* sv, int* si, ui
 }
 
 // One iteration of the fast scan (NV vectors per lane, d[j] = vector vfirst +
-// 32 j, there if bit j of `in`): a packed max tree per lane and a vote; vectors with a logit at or
-// over the threshold are queued, and the queue is worked off once it holds 32.
+// 32 j; past the segment's end -inf, which no threshold lets through): a packed max tree per lane
+// and a vote; vectors with a logit at or over the threshold are queued, and the queue is worked off
+// once it holds 32.
 template <int DT>
 __device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint4* st, uint32_t* qi, int& qn,
-                                          const uint4 (&d)[PPS_TRUNC_UNITS], unsigned in, const char* row,
-                                          int64_t vfirst, int h, int k) {
+                                          const uint4 (&d)[PPS_TRUNC_UNITS], const char* row, int64_t vfirst,
+                                          int h, int k) {
     constexpr int NV = PPS_TRUNC_UNITS;
     const int lane = threadIdx.x & 31;
+    // with no threshold yet (fewer than k usable tokens so far) a vector of nothing but -inf, a masked
+    // stretch of the vocabulary, still has none to offer
+    const float thr = fmaxf(C.thr, -FLT_MAX);
     unsigned vf = 0;
     if constexpr (DT == 1) {
-        const uint32_t tb = __float_as_uint(C.thr) >> 16;  // a bf16 value (or -inf) on bf16 rows
+        const uint32_t tb = __float_as_uint(thr) >> 16;  // a bf16 value on bf16 rows
         const uint32_t t2 = tb | (tb << 16);
         uint32_t mv[NV];
 #pragma unroll
@@ -484,14 +488,13 @@ __device__ __forceinline__ void topk_step(CandState& C, float* sv, int* si, uint
         float m = mv[0];
 #pragma unroll
         for (int j = 1; j < NV; ++j) m = fmaxf(m, mv[j]);
-        const bool hit = m >= C.thr;
+        const bool hit = m >= thr;
         if (!__any_sync(FULL, hit)) return;
         if (hit) {
 #pragma unroll
-            for (int j = 0; j < NV; ++j) vf |= (unsigned)(mv[j] >= C.thr) << j;
+            for (int j = 0; j < NV; ++j) vf |= (unsigned)(mv[j] >= thr) << j;
         }
     }
-    vf &= in;  // past the segment's end a vector of -inf reaches a threshold of -inf, but is not there to be read again
     const int n = __popc(vf);
     int off = n;
 #pragma unroll
@@ -527,24 +530,16 @@ __device__ __forceinline__ void topk_scan(CandState& C, float* sv, int* si, uint
     for (int64_t it = 0; it < n_it; ++it) {
         const int64_t vb = v0 + it * STEP + lane;
         uint4 d[NV];
-        unsigned in = (1u << NV) - 1u;  // which of the vectors exist
         if (v0 + (it + 1) * STEP <= vend) {
 #pragma unroll
             for (int j = 0; j < NV; ++j) d[j] = ldg_stream(p + 32 * j);
         } else {
-            in = 0;
 #pragma unroll
-            for (int j = 0; j < NV; ++j) {
-                d[j] = fill;
-                if (vb + 32 * j < vend) {
-                    d[j] = ldg_stream(p + 32 * j);
-                    in |= 1u << j;
-                }
-            }
+            for (int j = 0; j < NV; ++j) d[j] = vb + 32 * j < vend ? ldg_stream(p + 32 * j) : fill;
         }
         p += STEP;
         if (it == 0) C.thr = fmaxf(guess, seed_thr<DT>(d, k));
-        topk_step<DT>(C, sv, si, st, qi, qn, d, in, row, vb, h, k);
+        topk_step<DT>(C, sv, si, st, qi, qn, d, row, vb, h, k);
     }
     if (qn > 0) C = topk_flush<DT>(C, sv, si, st, qi, qn, row, h, k);
 }
