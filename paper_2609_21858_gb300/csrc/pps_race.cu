@@ -346,31 +346,34 @@ __device__ __forceinline__ uint64_t list_pack(float k, int i) { return ((uint64_
 
 // Merge one offer per lane (key ok, token oi; `valid` lanes only, below the
 // list's last entry) into the warp list by ranks: every entry counts the
-// entries before it, read from shared memory, and goes to the slot of its
+// offers before it, read from shared memory, an offer's lane also the list's entries
+// before it (a ballot per offer), and each goes to the slot of its
 // rank.  No lane waits for another's shuffle, where a bitonic sort and merge were
 // a chain of 20 of them (a K = 8 row of a one-sequence launch spent 10 us of its
 // 25 in its flushes; 64 sequences of the benchmark tree: 501 -> 488 us a step, of 8
-// non-identical proposals: 731 -> 704 us).  Lists without a spare entry record the smallest key left out.
-// `scratch`: 96 words of 64 bits of the warp's shared memory.
+// non-identical proposals: 731 -> 704 us; while every lane also read the whole list for its own offer,
+// rows of K = 32 took 15% longer than with the bitonic merge, V = 128256: 39 and 45 us, now 36).  Lists without a spare entry record the smallest key left out.
+// `scratch`: 64 words of 64 bits of the warp's shared memory.
 __device__ __forceinline__ void list_merge(WarpList& L, bool valid, float ok, int oi, int lane, uint64_t* scratch) {
-    uint64_t *s_offer = scratch, *s_list = scratch + 32, *s_out = scratch + 64;
+    uint64_t *s_offer = scratch, *s_out = scratch + 32;
     constexpr uint64_t kEmpty = (0xff800000ull << 32) | INT_MAX;  // list_pack(+inf, INT_MAX)
     const unsigned vm = __ballot_sync(FULL, valid);
     const int nb = __popc(vm);
     const uint64_t b = list_pack(ok, oi), l = list_pack(L.lk, L.li);
-    if (valid) s_offer[__popc(vm & ((1u << lane) - 1u))] = b;
-    s_list[lane] = l;
+    const int at = __popc(vm & ((1u << lane) - 1u));  // a valid lane's offer
+    if (valid) s_offer[at] = b;
     s_out[lane] = kEmpty;
     __syncwarp();
     int rl = lane, rb = 0;
-#pragma unroll 2
+#pragma unroll 4
     for (int j = 0; j < nb; ++j) {
         const uint64_t x = s_offer[j];
         rl += x < l;
         rb += x < b;
+        // the offer's own lane: the list's entries before it
+        const int before = 32 - __popc(__ballot_sync(FULL, x < l));
+        rb += j == at ? before : 0;
     }
-#pragma unroll 2
-    for (int j = 0; j < L.kp; ++j) rb += s_list[j] < b;
     const bool have = L.li != INT_MAX;
     if (have && rl < L.kp) s_out[rl] = l;
     if (valid && rb < L.kp) s_out[rb] = b;
