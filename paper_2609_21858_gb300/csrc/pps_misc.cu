@@ -218,8 +218,19 @@ __global__ void __launch_bounds__(256, 4) wm_score_kernel(const int32_t* __restr
                     v += at >= a && at < b ? A[u] : 0.0f;
                 }
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+                for (int o = 16; o > 2; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
+                // the four sums of 32 are added without loss, as the scan below adds its sums of 32:
+                // sums of up to 128 in fp32 alone left segments of 100 to 160 tokens a relative rms error
+                // of 3.2e-8, these 1.9e-8, the scan 2.2e-8 (6.6 10^6 tuples in texts of 38: 215 -> 218 us)
+                float lo = 0.0f;
+#pragma unroll
+                for (int o = 2; o > 0; o >>= 1) {
+                    const float ov = __shfl_xor_sync(FULL, v, o);
+                    if (o == 1) lo += __shfl_xor_sync(FULL, lo, o);
+                    ff_add(v, lo, ov);
+                }
                 ff_add(chi, clo, v);
+                clo += lo;
                 if (seg_end >= gend) break;  // stays open
                 s0 = seg_end;
                 flush();
