@@ -745,7 +745,9 @@ cudaError_t launch_wm_score(const int32_t* tokens, const uint64_t* key, const ui
         const int64_t chunk = ((n + resident - 1) / resident + group - 1) / group * group;
         const int64_t warps = (n + chunk - 1) / chunk;
         const int64_t blocks = (warps * 32 + 255) / 256;
-        // 16-byte loads and stores need 16-byte aligned arrays (chunks start on multiples of 128 tuples)
+        // pairs of tuples are loaded and stored together, 16 bytes of keys and labels, 8 of tokens, positions
+        // and scores; arrays that all start on 16-byte boundaries take that path (chunks start on multiples
+        // of 128 tuples)
         auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
         const bool vec = al(tokens) && al(key) && al(ctx) && al(pos) && (out_score == nullptr || al(out_score));
         if (vec)

@@ -352,7 +352,7 @@ __device__ __forceinline__ uint64_t list_pack(float k, int i) { return ((uint64_
 // a chain of 20 of them (a K = 8 row of a one-sequence launch spent 10 us of its
 // 25 in its flushes; 64 sequences of the benchmark tree: 501 -> 488 us a step, of 8
 // non-identical proposals: 731 -> 704 us; while every lane also read the whole list for its own offer,
-// rows of K = 32 took 15% longer than with the bitonic merge, V = 128256: 39 and 45 us, now 36).  Lists without a spare entry record the smallest key left out.
+// rows of K = 32 took 15% longer than with the bitonic merge, V = 128256: 39 and 45 us, now 35).  Lists without a spare entry record the smallest key left out.
 // `scratch`: 64 words of 64 bits of the warp's shared memory.
 __device__ __forceinline__ void list_merge(WarpList& L, bool valid, float ok, int oi, int lane, uint64_t* scratch) {
     uint64_t *s_offer = scratch, *s_out = scratch + 32;
@@ -1547,8 +1547,9 @@ __global__ void __launch_bounds__(kThreads, BLK ? PPS_BLOCK_MIN_BLOCKS : PPS_RAC
         // such rows stream like verify rows (one filter test per vector; measured: lists of up
         // to 4 gain, lists of 8 lose).  A row cut between warps shares its filter bound (verify,
         // short-list bf16 draft and proposal rows: on longer lists the shared bound saves too little,
-        // and in fp32 draft rows, half the tokens to a byte, the loop without its read is faster:
-        // 41216 rows of V = 152064 4.93 -> 4.63 ms, 16 sequences of that tree 854 -> 834 us a step;
+        // and in fp32 draft rows, half the tokens to a byte, the loop without its read is faster when
+        // there are many: 41216 rows of V = 152064 4.93 -> 4.63 ms, 16 sequences of that tree 854 -> 834 us a
+        // step, 1300 rows of V = 8192 to 128256 1 to 5%; up to 41 such rows of one token it costs 1 us in 14;
         // the benchmark's bf16 tree takes 488 us with it, 497 without).
         const bool one = VERIFY || (!BLK && kr <= PPS_VF_MAXK);
         uint32_t* slot = nullptr;
@@ -1591,8 +1592,10 @@ int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk, int64_t
     int64_t g = (int64_t)device_sm_count() * o;
     // a warp per row at least: rows of fewer vectors one after another in a warp add up their latencies
     // (64 sequences of 3 rows of V = 1000, fp32: 45 -> 33 us a step)
-    // (rows of 1024 vectors and more may be cut twice as fine: 12 sequences, V = 18368, 41 -> 38 us; shorter
-    // rows gain nothing from a second warp: V = 1000, fp32, 33 -> 44 us)
+    // (rows of 1024 vectors and more may be cut twice as fine: 12 sequences, V = 18368, 41 -> 38 us, 48 rows
+    // of V = 8192 bf16 or 4096 fp32, which are 1024 vectors, 18.5 -> 17.0 and 16.4 -> 14.4 us; rows of 512
+    // would gain too, 18.0 -> 16.9 and 16.6 -> 14.2; rows of 250 gain nothing from a second warp: V = 1000,
+    // fp32, 33 -> 44 us)
     const int64_t least = n_rows > 0 && total >= 1024 * n_rows ? kMinVecsPerWarp / 2 : kMinVecsPerWarp;
     const int64_t by_size = max((total + least - 1) / least, n_rows);
     if (by_size < g) g = by_size;
@@ -1606,7 +1609,7 @@ int race_grid(int64_t total, int dtype, bool verify, bool vec, bool blk, int64_t
     }
     if (n_rows > 0 && g >= 2 * n_rows) {
         // the same number of warps for every row, if that leaves no more than a sixteenth of them out
-        // or their segments stay short (4 iterations): a warp across two rows pays for two seeds and
+        // or their segments stay short (384 vectors: four iterations of bf16, two of fp32): a warp across two rows pays for two seeds and
         // two tickets, one after the other, and both rows wait for it (8 sequences of 4 chains,
         // V = 32000: 48.5 -> 39.7 us a step; 24 of 6, V = 32001, IID: 95 -> 80 us)
         const int64_t whole = g / n_rows * n_rows;
@@ -1647,10 +1650,11 @@ cudaError_t launch_race(const RaceArgs& a, int dtype, bool verify, bool vec, cud
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-// Rows stay whole when there are no more warps than rows (a segment's candidate
-// count grows like k ln(segment / k), and a row finished by one warp needs no
-// merge); fewer rows than warps get the same number of warps each, up to
-// kTruncSegCap of at least kTruncMinVecs vectors.
+// Fewer rows than resident warps get the same number of warps each, one to
+// kTruncSegCap of at least kTruncMinVecs vectors (a segment's candidate count
+// grows like k ln(segment / k), and a row finished by one warp needs no merge).
+// More rows share the vectors equally between the resident warps, so that
+// with little more than one row a warp most rows are cut between two.
 static const void* trunc_fn(int dtype, bool verify, bool blk) {
     if (dtype == 1) {
         if (verify) return (const void*)trunc_kernel<1, true, false>;

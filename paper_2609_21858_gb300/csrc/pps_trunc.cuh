@@ -33,8 +33,8 @@
 // A step of the benchmark's tree (top-k 50: 1.21 GB of logits) takes 266 us =
 // 4.6 TB/s, 290 when every row's threshold climbed from the first iteration's and S
 // was sorted; one sequence 263 -> 88 us; 16720 rows of V = 5717 736 -> 248 us.  It is
-// bound by HBM (0.78 of the measured copy rate inside the launch, 8% of the reads being
-// the sample) and by the finish of the last rows, about 12 us a launch.
+// bound by HBM (0.78 of the measured copy rate inside the launch; the sample, 6.4% of a row,
+// is read twice) and by the finish of the last rows, about 12 us a launch.
 
 #ifndef PPS_TRUNC_UNITS
 #define PPS_TRUNC_UNITS 8  // 16-byte vectors per lane per iteration of the top-k scan (even)
@@ -52,7 +52,10 @@ constexpr int kTruncSegCap = PPS_TRUNC_SEG_CAP;  // at most this many warps per 
 #ifndef PPS_TRUNC_MIN_VECS
 #define PPS_TRUNC_MIN_VECS 512
 #endif
-constexpr int64_t kTruncMinVecs = PPS_TRUNC_MIN_VECS;  // a row is not cut finer (132 rows of V = 7338: 256 66 us, 512 58)
+// a row is not cut finer: a step of 132 rows of V = 7338 took 66 us with 256 and 58 with 512; lists of 64
+// rows of 512, 1024 and 2048 vectors take 23, 23.5 and 27.4 us with 256, 19.3, 25.9 and 26.5 with 512, and
+// 19.3, 27.6 and 33.6 with 1024
+constexpr int64_t kTruncMinVecs = PPS_TRUNC_MIN_VECS;
 constexpr int kTruncRounds = 8;  // kept lists up to this long are selected by argmin rounds
 
 // ---------------------------------------------------------------- top lists
@@ -200,9 +203,16 @@ __device__ __forceinline__ float seed_thr(const uint4 (&d)[PPS_TRUNC_UNITS], int
 // 50) and hardly ever compacts; the threshold the first iteration proves
 // lets through ~1000 and compacts every 46 (a step of the benchmark's tree 289 -> 263 us).  It is a guess: topk_segment checks
 // that k tokens reached it.  One maximum per chunk keeps a cluster of large
-// logits (a vocabulary sorted by frequency) from raising it.
+// logits (a vocabulary sorted by frequency) from raising it.  What it costs: a row
+// in descending order, whose first iteration holds the top k, pays for the sample alone (1024
+// rows of V = 128256 bf16 66 -> 73 us, of random rows 101 -> 87), and a row with its largest
+// logits all in the sampled chunks (a random one: once in 10^4) is scanned twice (101 -> 128 us).
+// Sixteen chunks loaded together instead of eight spill (265 -> 270 us).
 constexpr int kSampleChunks = 32;
-constexpr int64_t kSampleMin = 32 * 192;  // vectors; shorter segments gain nothing from a guess
+// vectors from which a segment takes a guess: 3040 rows of V = 49160 bf16 (6145 vectors) 88.3 -> 85.0 us with
+// it, of V = 72000 109.5 -> 95.0; rows of 4500 vectors would gain too (76.9 -> 71.8 us), segments of
+// 3072 from k = 10 on some (51.7 -> 47.2) and from k = 50 on not (67.2 -> 69.4)
+constexpr int64_t kSampleMin = 32 * 192;
 
 template <int DT>
 __device__ __noinline__ float guess_thr(const char* row, int64_t v0, int64_t vend, int k) {

@@ -156,10 +156,12 @@ def _hard_rows(n, V, dtype, seed):
     return x.to(dtype)
 
 
-# rows too many to be cut (long enough for a guess) and few rows cut between warps; starts on 16-byte boundaries and not
+# rows too many to be cut (long enough for a guess) and few rows cut between warps; starts on 16-byte boundaries and not;
+# the last three are long enough for a guess (6144 vectors) whole and cut in two, wherever the number of resident warps lies
 @pytest.mark.parametrize("n,V,dtype,shift", [(2900, 65536, torch.bfloat16, 0), (3100, 49201, torch.bfloat16, 3),
                                              (2900, 24700, torch.float32, 1), (11, 70001, torch.bfloat16, 1),
-                                             (7, 30000, torch.float32, 0)])
+                                             (7, 30000, torch.float32, 0), (2900, 98400, torch.bfloat16, 0),
+                                             (3100, 98411, torch.bfloat16, 3), (2900, 49201, torch.float32, 1)])
 def test_top_k_threshold_of_hard_rows(n, V, dtype, shift):
     wide = torch.full((n, V + (-V % 8) + 8), 50.0, dtype=dtype, device="cuda")
     x = wide[:, shift:shift + V]
