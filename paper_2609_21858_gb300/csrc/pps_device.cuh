@@ -327,10 +327,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-#ifndef PPS_FILTER
-#define PPS_FILTER 0
-#endif
-#if PPS_FILTER == 0
 // 2^23 + (w >> 9) as fp32 bits from one mad.hi; cut 2^24 - 2, T scaled by 2^23
 constexpr float kFilterScaleLog2 = 23.0f;
 constexpr float kFilterCut = 16777214.0f;  // 2^24 - 2
@@ -339,16 +335,6 @@ __device__ __forceinline__ float filter_word(uint32_t w) {
     asm("mad.hi.u32 %0, %1, %2, %3;" : "=r"(bb) : "r"(w), "r"(1u << 23), "r"(0x4b000000u));
     return __uint_as_float(bb);
 }
-#else
-// 0x4b000000 | (w >> 8) as fp32 bits from one byte permute: 2^23 + (w >> 8) for
-// w < 2^31 and 2 (w >> 8) above; the token can be dropped when T + f <= 2^25 - 2
-// (T scaled by 2^25), and the fp32 sum errs by at most 2, so the cut is 2^25 - 4.
-// Below 2^31 the test drops only words with u < 3/4 - e_z, inside the safe
-// region u <= 1 - e_z.
-constexpr float kFilterScaleLog2 = 25.0f;
-constexpr float kFilterCut = 33554428.0f;  // 2^25 - 4
-__device__ __forceinline__ float filter_word(uint32_t w) { return __uint_as_float(__byte_perm(w, 0x4bu, 0x4321)); }
-#endif
 __device__ __forceinline__ float filter_sum(uint32_t w, float l, float c, float tz) {
     return ex2_approx(fmaf(l, c, tz)) + filter_word(w);
 }
