@@ -1033,49 +1033,6 @@ __device__ __forceinline__ double exact_key(uint64_t key, uint64_t ctx, uint32_t
     }
 }
 
-// The `take` <= 32 smallest of the warp's 32 x N entries (d, id) in order: lane m receives the m-th.
-template <int N>
-__device__ __forceinline__ void select_exact(double (&d)[N], int (&id)[N], int take, int lane, double& dk, int& li) {
-    dk = (double)INFINITY;
-    li = INT_MAX;
-    for (int m = 0; m < take; ++m) {
-        double bd = d[0];
-        int bi = id[0], bt = 0;
-#pragma unroll
-        for (int t = 1; t < N; ++t)
-            if (lex_less_d(d[t], id[t], bd, bi)) {
-                bd = d[t];
-                bi = id[t];
-                bt = t;
-            }
-        double wd = bd;
-        int wi = bi, wl = lane;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            const double od = __shfl_xor_sync(FULL, wd, off);
-            const int oi = __shfl_xor_sync(FULL, wi, off);
-            const int ol = __shfl_xor_sync(FULL, wl, off);
-            if (lex_less_d(od, oi, wd, wi)) {
-                wd = od;
-                wi = oi;
-                wl = ol;
-            }
-        }
-        if (lane == m) {
-            dk = wd;
-            li = wi;
-        }
-        if (lane == wl) {
-#pragma unroll
-            for (int t = 0; t < N; ++t)
-                if (t == bt) {
-                    d[t] = (double)INFINITY;
-                    id[t] = INT_MAX;
-                }
-        }
-    }
-}
-
 // Exact finish of a row whose list could not prove itself complete: tokens
 // crowd its k-th key tau within the error bounds and the 32-entry list has no
 // room left to hold them (always the case for k = 32 on a full list).  One
@@ -1154,8 +1111,47 @@ __device__ __noinline__ bool rescan_row(const RaceArgs& a, int64_t r, float tau,
             d[t] = exact_key<BLK>(key, ctx, pos, id[t], logit_at<DT>(a, r, id[t]), a.T, bk);
         }
     }
-    nvalid = min(n, 32);
-    select_exact<3>(d, id, nvalid, lane, dk, li);
+    // the min(n, 32) smallest in order: lane m receives the m-th
+    dk = (double)INFINITY;
+    li = INT_MAX;
+    const int take = min(n, 32);
+    for (int m = 0; m < take; ++m) {
+        double bd = d[0];
+        int bi = id[0], bt = 0;
+#pragma unroll
+        for (int t = 1; t < 3; ++t)
+            if (lex_less_d(d[t], id[t], bd, bi)) {
+                bd = d[t];
+                bi = id[t];
+                bt = t;
+            }
+        double wd = bd;
+        int wi = bi, wl = lane;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const double od = __shfl_xor_sync(FULL, wd, off);
+            const int oi = __shfl_xor_sync(FULL, wi, off);
+            const int ol = __shfl_xor_sync(FULL, wl, off);
+            if (lex_less_d(od, oi, wd, wi)) {
+                wd = od;
+                wi = oi;
+                wl = ol;
+            }
+        }
+        if (lane == m) {
+            dk = wd;
+            li = wi;
+        }
+        if (lane == wl) {
+#pragma unroll
+            for (int t = 0; t < 3; ++t)
+                if (t == bt) {
+                    d[t] = (double)INFINITY;
+                    id[t] = INT_MAX;
+                }
+        }
+    }
+    nvalid = take;
     return true;
 }
 
