@@ -21,9 +21,14 @@ import torch
 from . import pps
 
 
-def _as_stored(x, mine, n: int) -> bool:
-    """Whether x is n values of mine's dtype on its device, so that a copy into it changes nothing but the place."""
-    return isinstance(x, torch.Tensor) and x.dtype is mine.dtype and x.device == mine.device and x.shape == (n,)
+def _plain_roots(key, ctx, pos, n: int, device: int) -> bool:
+    """Whether the root identities are n keys, labels and positions of the dtypes the builders store, on
+    their device (its index, -1: the CPU): then plain copies write them."""
+    T = torch.Tensor
+    return (isinstance(key, T) and isinstance(ctx, T) and isinstance(pos, T)
+            and key.dtype is torch.int64 and ctx.dtype is torch.int64 and pos.dtype is torch.int32
+            and key.get_device() == ctx.get_device() == pos.get_device() == device
+            and key.dim() == ctx.dim() == pos.dim() == 1 and key.numel() == ctx.numel() == pos.numel() == n)
 
 
 class TreeBuilder:
@@ -58,10 +63,13 @@ class TreeBuilder:
         self.row_pos = torch.zeros(self.row_key.numel(), **i32)
         self.row_k = torch.zeros(self.row_key.numel(), **i32)
         self.roots = self.seq_off[:-1].long()
+        self._device = self.roots.get_device()
         self.ws = pps.workspace(n_seq * K, 0, dev)
         # what every run hands on per depth, and the root nodes' identities, as views made once
         self._ids = [tuple(t[self.rows(d)] for t in (self.row_key, self.row_ctx, self.row_pos, self.row_k))
                      for d in range(gamma + 1)]
+        self._next = [dict(zip(("key", "ctx", "pos", "k"), ids)) for ids in self._ids[1:]]
+        self._nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
         self._out = [dict(tok=self.draft_tok[s], key=None, mult=self.draft_mult[s], ndist=self.draft_ndist[s],
                           samples=None) for s in map(self.rows, range(gamma))]
         self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
@@ -73,12 +81,13 @@ class TreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_list (IID) and one pps_tree_expand."""
         K = self.K
-        nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
-        for mine, root, node, x in zip(self._ids[0], self._root, nodes.values(), (root_key, root_ctx, root_pos)):
-            if _as_stored(x, mine, self.n_seq):
+        roots = (root_key, root_ctx, root_pos)
+        if _plain_roots(*roots, self.n_seq, self._device):
+            for mine, root, x in zip(self._ids[0], self._root, roots):
                 mine.copy_(x)
                 root.copy_(x)
-            else:  # a scalar or one root for all; the write by index refuses any other dtype, device or length
+        else:  # scalars or one root for all; the writes by index refuse any other dtype, device or length
+            for mine, node, x in zip(self._ids[0], self._nodes.values(), roots):
                 mine[:] = x
                 node[self.roots] = x
         self._ids[0][3].fill_(K)
@@ -87,8 +96,8 @@ class TreeBuilder:
             out = self._out[d]
             pps.draft_list(draft_logits(d, key, ctx, pos), key, ctx, pos, K, row_k=k, mode=pps.IID,
                            temperature=temperature, ws=self.ws, out=out, top_k=top_k, top_p=top_p, stream=stream)
-            nxt = dict(zip(("key", "ctx", "pos", "k"), self._ids[d + 1]))
-            pps.tree_expand(K, self.gamma, d, out, key, ctx, pos, k, nxt, self.child_node, nodes, stream=stream)
+            pps.tree_expand(K, self.gamma, d, out, key, ctx, pos, k, self._next[d], self.child_node, self._nodes,
+                            stream=stream)
         return self
 
     def verify(self, p_logits, temperature: float = 1.0, top_k: int = 0, top_p: float = 1.0, ws=None, out=None,
@@ -148,9 +157,14 @@ class HeteroTreeBuilder:
         self.row_block = torch.arange(B, **i32).repeat(n_seq * gamma)
         self.draft_tok = torch.full((nr,), -1, **i32)
         self.roots = self.seq_off[:-1].long()
+        self._device = self.roots.get_device()
         self.ws = pps.workspace(n_seq * B, 0, dev)
         self._ids = [tuple(t[self.rows(d)] for t in (self.row_key, self.row_ctx, self.row_pos, self.row_owner))
                      for d in range(gamma)]
+        self._first = [t.view(n_seq, B) for t in self._ids[0][:3]]
+        self._next = [dict(zip(("key", "ctx", "pos", "owner"), ids)) for ids in self._ids[1:]] + [None]
+        self._nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
+        self._lists = dict(tok=self.list_tok, ndist=self.list_nd, child=self.child_node)
         self._blk_tok = [(self.row_block[s], self.draft_tok[s]) for s in map(self.rows, range(gamma))]
         self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
 
@@ -162,13 +176,13 @@ class HeteroTreeBuilder:
             top_p: float = 1.0, stream=None):
         """Draft the trees: per depth one pps_draft_hetero and one pps_hetero_expand."""
         B = self.B
-        lists = dict(tok=self.list_tok, ndist=self.list_nd, child=self.child_node)
-        nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
-        for mine, root, node, x in zip(self._ids[0], self._root, nodes.values(), (root_key, root_ctx, root_pos)):
-            if _as_stored(x, mine, self.n_seq):
-                mine.view(self.n_seq, B).copy_(x[:, None].expand(-1, B))
+        roots = (root_key, root_ctx, root_pos)
+        if _plain_roots(*roots, self.n_seq, self._device):
+            for mine, root, x in zip(self._first, self._root, roots):
+                mine.copy_(x[:, None])
                 root.copy_(x)
-            else:  # the write by index refuses another dtype, device or length
+        else:  # the writes by index refuse any other dtype, device or length
+            for mine, node, x in zip(self._ids[0], self._nodes.values(), roots):
                 mine[:] = x.repeat_interleave(B)
                 node[self.roots] = x
         self._ids[0][3].zero_()
@@ -177,8 +191,8 @@ class HeteroTreeBuilder:
             blk, tok = self._blk_tok[d]
             pps.draft_hetero(draft_logits(d, key, ctx, pos, blk), key, ctx, pos, blk, B, temperature=temperature,
                              ws=self.ws, out_tok=tok, stream=stream, top_k=top_k, top_p=top_p)
-            nxt = dict(zip(("key", "ctx", "pos", "owner"), self._ids[d + 1])) if d + 1 < self.gamma else None
-            pps.hetero_expand(B, self.gamma, d, tok, key, ctx, pos, owner, nxt, lists, nodes, stream=stream)
+            pps.hetero_expand(B, self.gamma, d, tok, key, ctx, pos, owner, self._next[d], self._lists, self._nodes,
+                              stream=stream)
         return self
 
     def verify(self, p_logits, temperature: float = 1.0, top_k: int = 0, top_p: float = 1.0, ws=None, out=None,
