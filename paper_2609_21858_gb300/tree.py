@@ -72,7 +72,7 @@ class TreeBuilder:
         self._nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
         self._out = [dict(tok=self.draft_tok[s], key=None, mult=self.draft_mult[s], ndist=self.draft_ndist[s],
                           samples=None) for s in map(self.rows, range(gamma))]
-        self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
+        self._places = list(self._ids[0][:3]) + [t.view(n_seq, N1)[:, 0] for t in self._nodes.values()]
 
     def rows(self, d: int) -> slice:
         return slice(self.depth_start[d], self.depth_start[d] + self.n_seq * self.width[d])
@@ -82,10 +82,8 @@ class TreeBuilder:
         """Draft the trees: per depth one pps_draft_list (IID) and one pps_tree_expand."""
         K = self.K
         roots = (root_key, root_ctx, root_pos)
-        if _plain_roots(*roots, self.n_seq, self._device):
-            for mine, root, x in zip(self._ids[0], self._root, roots):
-                mine.copy_(x)
-                root.copy_(x)
+        if _plain_roots(root_key, root_ctx, root_pos, self.n_seq, self._device):
+            torch._foreach_copy_(self._places, roots + roots)
         else:  # scalars or one root for all; the writes by index refuse any other dtype, device or length
             for mine, node, x in zip(self._ids[0], self._nodes.values(), roots):
                 mine[:] = x
@@ -161,12 +159,12 @@ class HeteroTreeBuilder:
         self.ws = pps.workspace(n_seq * B, 0, dev)
         self._ids = [tuple(t[self.rows(d)] for t in (self.row_key, self.row_ctx, self.row_pos, self.row_owner))
                      for d in range(gamma)]
-        self._first = [t.view(n_seq, B) for t in self._ids[0][:3]]
         self._next = [dict(zip(("key", "ctx", "pos", "owner"), ids)) for ids in self._ids[1:]] + [None]
         self._nodes = dict(key=self.node_key, ctx=self.node_ctx, pos=self.node_pos)
         self._lists = dict(tok=self.list_tok, ndist=self.list_nd, child=self.child_node)
         self._blk_tok = [(self.row_block[s], self.draft_tok[s]) for s in map(self.rows, range(gamma))]
-        self._root = [t.view(n_seq, N1)[:, 0] for t in (self.node_key, self.node_ctx, self.node_pos)]
+        self._places = ([t.view(n_seq, B) for t in self._ids[0][:3]]
+                        + [t.view(n_seq, N1)[:, :1] for t in self._nodes.values()])
 
     def rows(self, d: int) -> slice:
         n = self.n_seq * self.B
@@ -177,10 +175,8 @@ class HeteroTreeBuilder:
         """Draft the trees: per depth one pps_draft_hetero and one pps_hetero_expand."""
         B = self.B
         roots = (root_key, root_ctx, root_pos)
-        if _plain_roots(*roots, self.n_seq, self._device):
-            for mine, root, x in zip(self._first, self._root, roots):
-                mine.copy_(x[:, None])
-                root.copy_(x)
+        if _plain_roots(root_key, root_ctx, root_pos, self.n_seq, self._device):
+            torch._foreach_copy_(self._places, [x[:, None] for x in roots] * 2)
         else:  # the writes by index refuse any other dtype, device or length
             for mine, node, x in zip(self._ids[0], self._nodes.values(), roots):
                 mine[:] = x.repeat_interleave(B)
