@@ -716,9 +716,9 @@ static cudaError_t launch_gemm(const CUtensorMap& tA, const CUtensorMap& tB, con
 // The schedule: MB row blocks x S vocabulary slices, S = SMs / MB (at least 1, at most NT), so that
 // every SM has a CTA.  With few row blocks the pass is bound by reading the weights once from HBM,
 // which takes the whole chip: the two launches of one sequence (41 rows of d = 4096, 33 of d = 2048,
-// V = 128256: 1.58 GB) take 303 us = 5.2 TB/s, 1131 us on 16 slices.  A single row block takes
+// V = 128256: 1.58 GB) take 309 us = 5.1 TB/s, 1131 us on 16 slices.  A single row block takes
 // 128-column tiles where they shorten the longest slice (501 tiles of 256 on 152 slices: four, or seven
-// halves; 319 -> 303 us for one sequence, 328 -> 320 us for the 123 rows of three); where they do not
+// halves; in one run 319 -> 303 us for one sequence, 328 -> 320 us for the 123 rows of three); where they do not
 // (V = 66624, 117 rows: 239 against 254 us) and with more row blocks, where the tensor cores count, 256.
 // (One equal run of tiles per SM across row blocks, walked in phase, was slower than whole slices: 2642
 // against 2516 us for 64 sequences, although it uses 152 SMs instead of 136 and 147.)
