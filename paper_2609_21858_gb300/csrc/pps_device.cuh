@@ -14,6 +14,7 @@
 // an error bounded by key_err_bound(); pairs closer than the sum of their
 // bounds are re-ordered with the fp64 key s.
 #pragma once
+#include <cfloat>
 #include <cstdint>
 #include <cuda_runtime.h>
 #include "pps_internal.h"
@@ -341,8 +342,10 @@ __device__ __forceinline__ float filter_sum(uint32_t w, float l, float c, float 
 __device__ __forceinline__ bool filter_pass(uint32_t w, float l, float c, float tz) {
     return filter_sum(w, l, c, tz) >= kFilterCut;
 }
+// A list full of +inf logits has theta = -inf.  Another +inf logit may still enter it, by its
+// smaller index, so tz stays finite: it passes then, where inf - inf would drop it.
 __device__ __forceinline__ float filter_tz(float theta) {
-    return theta + (kFilterMargin + kLog2Ln2 + kFilterScaleLog2);
+    return fmaxf(theta + (kFilterMargin + kLog2Ln2 + kFilterScaleLog2), -FLT_MAX);
 }
 
 // packed bf16 max (a NaN half yields the other operand's half)

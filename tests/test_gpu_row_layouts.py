@@ -113,3 +113,33 @@ def test_lists_of_rows_cut_between_many_warps(n, V, dtype, where):
         want = oracle.draft_rows(x.float().cpu().numpy(), *ids, K, mode=mode)
         compare_draft({k: v.cpu().numpy() for k, v in d.items()}, want)
     assert int(status.item()) == 0
+
+
+# +inf logits win, the lowest index first, however many there are: more than a list holds, met by the
+# lanes and warps of a row in another order than that of their indexes
+@pytest.mark.parametrize("dtype,offset,pad", [(BF, 0, 0), (BF, 1, 1), (F32, 0, 0), (F32, 3, 2)])
+@pytest.mark.parametrize("V,many", [(700, 20), (700, 200), (20000, 200), (20000, 3000), (128256, 4000)])
+def test_rows_with_many_infinite_logits(V, many, dtype, offset, pad):
+    n = 24
+    rng = np.random.default_rng(V + many)
+    x = rng.normal(0, 2.5, (n, V)).astype(np.float32)
+    for r in range(n):
+        x[r, rng.choice(V, many, replace=False)] = np.inf
+    x = torch.as_tensor(x).to(dtype).cuda()
+    ids = (rng.integers(0, 2 ** 64, n, dtype=np.uint64), rng.integers(0, 2 ** 64, n, dtype=np.uint64),
+           rng.integers(0, 2 ** 31, n, dtype=np.uint32))
+    dev = tuple(torch.as_tensor(a.view(t)).cuda() for a, t in zip(ids, (np.int64, np.int64, np.int32)))
+    y = _placed(x, offset, pad)
+    lowest = np.stack([np.nonzero(row == np.inf)[0][:32] for row in x.float().cpu().numpy()])
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    for kw in ({}, {"top_k": 50}):
+        for K in (1, 4, 8, 16):
+            d = pps.draft_list(y, *dev, K, status=status, **kw)
+            assert np.array_equal(d["tok"].cpu().numpy(), lowest[:, :K]), (K, kw)
+        assert np.array_equal(_verify(y, dev, status=status, **kw)["winner"].cpu().numpy(), lowest[:, 0]), kw
+        blk = torch.arange(n, dtype=torch.int32, device="cuda") % 5
+        x1 = pps.draft_hetero(y, *dev, blk, 5, status=status, **kw)
+        assert np.array_equal(x1.cpu().numpy(), lowest[:, 0]), kw
+    assert int(status.item()) == 0
+    want = oracle.draft_rows(x.float().cpu().numpy(), *ids, 16)
+    assert np.array_equal(want["tok"], lowest[:, :16])
